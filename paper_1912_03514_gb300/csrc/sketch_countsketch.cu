@@ -2,38 +2,139 @@
 //     SA[h(j), :] += s(j) · A[j, :],   j = 0 … n−1.
 //
 // Instead of scattering rows of A into SA with atomics, the rows are bucketed
-// by h once (a counting sort of n 32-bit keys: ~4 B/row of extra traffic) and
-// one thread block then owns each output row h and streams its rows of A in
-// ascending j.  A is read exactly once, in whole coalesced rows, every output
-// row is written exactly once (no memset, no atomics on SA), and the sum order
-// is fixed, so SA is bit-reproducible.
+// by h once (a counting sort of n 32-bit keys: ~12 B/row of extra traffic) and
+// thread blocks then own output rows h and stream their rows of A in
+// ascending j.  A is read exactly once, in coalesced segments, no atomic
+// touches SA, and the sum order is fixed, so SA is bit-reproducible.
+//
+// Counting sort: the n rows are cut into at most kMaxChunks chunks, one block
+// each, which counts its rows per bucket in shared memory and stores the m
+// counts; the scatter pass reads every chunk's counts, so that a block knows
+// where its rows of each bucket begin without a global atomic, and the chunk
+// boundaries inside a bucket are known too (`start`).  At 262144×1024, m = 588:
+// 4 µs to count and 11 µs to scatter, where one global counter per bucket took
+// 34 and 35 µs (446 atomics on each of 588 words, ≈ 76 ns apiece).  Above
+// kHistMaxM buckets the counts outgrow a block and few rows meet on a counter:
+// that range keeps the global ones.
 #include "internal.h"
 
 namespace mihs {
 
 namespace {
 
+constexpr int kMaxChunks = 64;     // the scatter pass reads chunks × m counts in every block
+constexpr int kChunkRows = 2048;   // fewest rows worth a chunk
+constexpr int kHistMaxM = 8192;    // bucket counters of a chunk in shared memory (32 KB)
+constexpr int kSortThreads = 1024;
 constexpr int kGatherThreads = 256;
 constexpr int kSortCap = 8192;  // bucket entries sorted in shared memory
 // Rows loaded before they are added (16-byte loads in flight per thread):
 // 4 left the gather bound by load latency (55 % of DRAM bandwidth).
 constexpr int kRowsInFlight = 8;
 
-// h(j) = ⌊w0·m/2³²⌋, s(j) = + if w1 even; Philox counter (j, 0, 1, 0).
-__global__ void cs_hash_kernel(int n, uint32_t m, uint32_t k0, uint32_t k1,
-                               int* __restrict__ code, int* __restrict__ counts) {
-  const int j = blockIdx.x * blockDim.x + threadIdx.x;
-  if (j >= n) return;
+// h(j) = ⌊w0·m/2³²⌋, s(j) = + if w1 even; Philox counter (j, 0, 1, 0).  The
+// sign travels in bit 31.
+__device__ __forceinline__ int cs_code(int j, uint32_t m, uint32_t k0, uint32_t k1) {
   const uint4 w = philox4x32_10(make_uint4((uint32_t)j, 0u, kTagCountSketch, 0u), k0, k1);
   const int h = (int)(((uint64_t)w.x * m) >> 32);
-  const int neg = (int)(w.y & 1u);
-  code[j] = h | (neg ? (int)0x80000000 : 0);  // the sign travels in bit 31
-  atomicAdd(counts + h, 1);
+  return h | ((w.y & 1u) ? (int)0x80000000 : 0);
 }
 
-// Exclusive scan of counts[0..m) → offsets[0..m], cursor = offsets (one block).
-__global__ void __launch_bounds__(1024) cs_scan_kernel(const int* __restrict__ counts, int m,
-                                                       int* __restrict__ offsets,
+// Counts of one chunk: code[j] for its rows and hist[chunk][h].
+__global__ void __launch_bounds__(kSortThreads)
+cs_count_kernel(int n, int m, int rows, uint32_t k0, uint32_t k1, int* __restrict__ code, int* __restrict__ hist) {
+  extern __shared__ int cnt[];
+  for (int h = threadIdx.x; h < m; h += kSortThreads) cnt[h] = 0;
+  __syncthreads();
+  const long long j1 = min((long long)n, (long long)(blockIdx.x + 1) * rows);
+  for (long long j = (long long)blockIdx.x * rows + threadIdx.x; j < j1; j += kSortThreads) {
+    const int c = cs_code((int)j, (uint32_t)m, k0, k1);
+    code[j] = c;
+    atomicAdd(cnt + (c & 0x7fffffff), 1);
+  }
+  __syncthreads();
+  for (int h = threadIdx.x; h < m; h += kSortThreads) hist[(size_t)blockIdx.x * m + h] = cnt[h];
+}
+
+// start[chunk][h] = where the chunk's rows of bucket h begin in the list, and
+// list[...] = j | (sign << 31) for its rows (the order inside a chunk's share
+// of a bucket is fixed later).  Every block sums all chunks' counts itself:
+// chunks · m words from L2 instead of one more launch.
+__global__ void __launch_bounds__(kSortThreads)
+cs_scatter_kernel(int n, int m, int rows, const int* __restrict__ code, const int* __restrict__ hist,
+                  int* __restrict__ start, int* __restrict__ list) {
+  extern __shared__ int cursor[];
+  __shared__ int wsum[kSortThreads / 32];
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const int chunks = gridDim.x, mine = blockIdx.x;
+  // The chunk's first codes, loaded while the counts are summed.
+  const long long j0 = (long long)mine * rows + threadIdx.x;
+  const long long j1 = min((long long)n, (long long)(mine + 1) * rows);
+  constexpr int kAhead = 4;
+  int ahead[kAhead];
+#pragma unroll
+  for (int u = 0; u < kAhead; ++u) ahead[u] = j0 + u * kSortThreads < j1 ? __ldg(code + j0 + u * kSortThreads) : 0;
+  int carry = 0;
+  for (int base = 0; base < m; base += kSortThreads) {
+    const int h = base + threadIdx.x;
+    int total = 0, before = 0;
+    if (h < m) {
+      for (int c0 = 0; c0 < chunks; c0 += 32) {  // 32 loads in flight
+        int v[32];
+#pragma unroll
+        for (int u = 0; u < 32; ++u) v[u] = c0 + u < chunks ? __ldg(hist + (size_t)(c0 + u) * m + h) : 0;
+#pragma unroll
+        for (int u = 0; u < 32; ++u) {
+          total += v[u];
+          before += c0 + u < mine ? v[u] : 0;
+        }
+      }
+    }
+    int inc = total;  // inclusive scan over the block's buckets
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+      const int t = __shfl_up_sync(0xffffffffu, inc, o);
+      if (lane >= o) inc += t;
+    }
+    if (lane == 31) wsum[warp] = inc;
+    __syncthreads();
+    int pre = 0, all = 0;
+#pragma unroll
+    for (int w = 0; w < kSortThreads / 32; ++w) {
+      const int t = wsum[w];
+      pre += w < warp ? t : 0;
+      all += t;
+    }
+    if (h < m) {
+      const int pos = carry + pre + inc - total + before;
+      cursor[h] = pos;
+      start[(size_t)mine * m + h] = pos;
+    }
+    carry += all;
+    __syncthreads();
+  }
+  auto place = [&](long long j, int c) {
+    const int pos = atomicAdd(cursor + (c & 0x7fffffff), 1);
+    list[pos] = (int)j | (c & (int)0x80000000);
+  };
+#pragma unroll
+  for (int u = 0; u < kAhead; ++u)
+    if (j0 + u * kSortThreads < j1) place(j0 + u * kSortThreads, ahead[u]);
+  for (long long j = j0 + kAhead * kSortThreads; j < j1; j += kSortThreads) place(j, code[j]);
+}
+
+// More than kHistMaxM buckets: one global counter per bucket (few rows share one).
+__global__ void cs_hash_global_kernel(int n, uint32_t m, uint32_t k0, uint32_t k1, int* __restrict__ code,
+                                      int* __restrict__ counts) {
+  const int j = blockIdx.x * blockDim.x + threadIdx.x;
+  if (j >= n) return;
+  const int c = cs_code(j, m, k0, k1);
+  code[j] = c;
+  atomicAdd(counts + (c & 0x7fffffff), 1);
+}
+
+// Exclusive scan of counts[0..m) → start, cursor (one block).
+__global__ void __launch_bounds__(1024) cs_scan_kernel(const int* __restrict__ counts, int m, int* __restrict__ start,
                                                        int* __restrict__ cursor) {
   __shared__ int buf[1024];
   __shared__ int carry;
@@ -52,153 +153,230 @@ __global__ void __launch_bounds__(1024) cs_scan_kernel(const int* __restrict__ c
     }
     if (i < m) {
       const int ex = carry + buf[threadIdx.x] - v;
-      offsets[i] = ex;
+      start[i] = ex;
       cursor[i] = ex;
     }
     __syncthreads();
     if (threadIdx.x == 1023) carry += buf[1023];
     __syncthreads();
   }
-  if (threadIdx.x == 0) offsets[m] = carry;
 }
 
-// list[offsets[h] + k] = j | (sign << 31)  (order within a bucket is fixed later)
-__global__ void cs_scatter_kernel(int n, const int* __restrict__ code, int* __restrict__ cursor,
-                                  int* __restrict__ list) {
+__global__ void cs_scatter_global_kernel(int n, const int* __restrict__ code, int* __restrict__ cursor,
+                                         int* __restrict__ list) {
   const int j = blockIdx.x * blockDim.x + threadIdx.x;
   if (j >= n) return;
   const int c = code[j];
-  const int h = c & 0x7fffffff;
-  const int pos = atomicAdd(cursor + h, 1);
+  const int pos = atomicAdd(cursor + (c & 0x7fffffff), 1);
   list[pos] = j | (c & (int)0x80000000);
 }
 
 __device__ __forceinline__ int entry_row(int e) { return e & 0x7fffffff; }
 __device__ __forceinline__ float entry_sign(int e) { return e < 0 ? -1.f : 1.f; }
 
-// One block per output row h: sort the bucket by j, then SA[h] = Σ s(j) A[j].
+// One block per (chunk range z, output row h, column slice of 4·CT columns):
+// sort its list entries by j, then Σ s(j) A[j] over them.  The 256 threads are
+// CT column groups (16 bytes each) × 256/CT row groups, which take every
+// 256/CT-th entry and are added in order at the end.
+//
+// Memory-bound: 4·n·d bytes.  Two things cost beyond them.  A row is read in
+// one piece where a block is wide enough (CT covers d up to 1024 columns): at
+// 262144×1024 slices of 64 / 128 / 256 / 512 / 1024 columns took 311 / 233 /
+// 200 / 184 / 171 µs, the random row segments costing DRAM locality.  And one
+// block per bucket, all 588 resident at once, ran as long as the fullest
+// bucket (180 µs); a bucket cut into chunk ranges (ks = 3 there) ends evenly:
+// 171 µs, 6.28 TB/s, 0.93 of the measured copy.
+template <int CT>
 __global__ void __launch_bounds__(kGatherThreads)
-cs_gather_kernel(const float* __restrict__ A, int d, long long lda,
-                 const int* __restrict__ offsets, const int* __restrict__ list, int m,
-                 float* __restrict__ SA, long long ldsa) {
+cs_gather_kernel(const float* __restrict__ A, int n, int d, long long lda, const int* __restrict__ start,
+                 const int* __restrict__ list, int m, int chunks, int ks, int slices, float* __restrict__ out,
+                 long long ldo, int vec_out) {
+  constexpr int RG = kGatherThreads / CT;
   __shared__ int keys[kSortCap];
-  for (int h = blockIdx.x; h < m; h += gridDim.x) {
-    const int beg = offsets[h], cnt = offsets[h + 1] - beg;
-    const bool sorted = cnt <= kSortCap;
-    if (sorted) {
-      int np2 = 1;
-      while (np2 < cnt) np2 <<= 1;
-      for (int e = threadIdx.x; e < np2; e += kGatherThreads)
-        keys[e] = e < cnt ? list[beg + e] : 0x7fffffff;
-      __syncthreads();
-      // bitonic sort by row index (bit 31 carries the sign, so sort on j)
-      for (int k = 2; k <= np2; k <<= 1) {
-        for (int jj = k >> 1; jj > 0; jj >>= 1) {
-          for (int e = threadIdx.x; e < np2; e += kGatherThreads) {
-            const int p = e ^ jj;
-            if (p > e) {
-              const int a = keys[e], b = keys[p];
-              const bool up = (e & k) == 0;
-              const bool gt = (a & 0x7fffffff) > (b & 0x7fffffff);
-              if (gt == up) {
-                keys[e] = b;
-                keys[p] = a;
-              }
+  __shared__ float4 red[RG > 1 ? kGatherThreads : 1];
+  const long long unit = blockIdx.x;
+  const int slice = (int)(unit % slices);
+  const long long zh = unit / slices;
+  const int h = (int)(zh % m), z = (int)(zh / m);
+  const int z0 = (int)((long long)z * chunks / ks), z1 = (int)((long long)(z + 1) * chunks / ks);
+  const int beg = start[(size_t)z0 * m + h];
+  const int end = z1 < chunks ? start[(size_t)z1 * m + h] : (h + 1 < m ? start[h + 1] : n);
+  const int cnt = end - beg;
+  const bool sorted = cnt <= kSortCap;
+  if (sorted) {
+    int np2 = 1;
+    while (np2 < cnt) np2 <<= 1;
+    for (int e = threadIdx.x; e < np2; e += kGatherThreads) keys[e] = e < cnt ? list[beg + e] : 0x7fffffff;
+    __syncthreads();
+    // bitonic sort by row index (bit 31 carries the sign, so sort on j)
+    for (int k = 2; k <= np2; k <<= 1) {
+      for (int jj = k >> 1; jj > 0; jj >>= 1) {
+        for (int e = threadIdx.x; e < np2; e += kGatherThreads) {
+          const int p = e ^ jj;
+          if (p > e) {
+            const int a = keys[e], b = keys[p];
+            const bool up = (e & k) == 0;
+            const bool gt = (a & 0x7fffffff) > (b & 0x7fffffff);
+            if (gt == up) {
+              keys[e] = b;
+              keys[p] = a;
             }
           }
-          __syncthreads();
         }
+        __syncthreads();
       }
     }
-    // Each thread owns float4 column groups q = tid + 256·c.
-    for (int q0 = 0; 4 * q0 < d; q0 += kGatherThreads) {
-      const int q = q0 + threadIdx.x;
-      const int col = 4 * q;
-      float4 acc = make_float4(0.f, 0.f, 0.f, 0.f);
-      if (col < d) {
-        const bool full = col + 4 <= d;
-        int e = 0;
-        for (; e + kRowsInFlight <= cnt; e += kRowsInFlight) {
-          int en[kRowsInFlight];
-          float4 a[kRowsInFlight];
-#pragma unroll
-          for (int u = 0; u < kRowsInFlight; ++u) en[u] = sorted ? keys[e + u] : list[beg + e + u];
-#pragma unroll
-          for (int u = 0; u < kRowsInFlight; ++u) {
-            const float* row = A + (long long)entry_row(en[u]) * lda + col;
-            if (full) {
-              a[u] = __ldcs(reinterpret_cast<const float4*>(row));
-            } else {
-              a[u] = make_float4(row[0], col + 1 < d ? row[1] : 0.f, col + 2 < d ? row[2] : 0.f, 0.f);
-            }
-          }
-#pragma unroll
-          for (int u = 0; u < kRowsInFlight; ++u) {
-            const float sg = entry_sign(en[u]);
-            acc.x = fmaf(sg, a[u].x, acc.x);
-            acc.y = fmaf(sg, a[u].y, acc.y);
-            acc.z = fmaf(sg, a[u].z, acc.z);
-            acc.w = fmaf(sg, a[u].w, acc.w);
-          }
-        }
-        for (; e < cnt; ++e) {
-          const int en = sorted ? keys[e] : list[beg + e];
-          const float* row = A + (long long)entry_row(en) * lda + col;
-          const float sg = entry_sign(en);
-          float4 a;
-          if (full) {
-            a = __ldcs(reinterpret_cast<const float4*>(row));
-          } else {
-            a = make_float4(row[0], col + 1 < d ? row[1] : 0.f, col + 2 < d ? row[2] : 0.f, 0.f);
-          }
-          acc.x = fmaf(sg, a.x, acc.x);
-          acc.y = fmaf(sg, a.y, acc.y);
-          acc.z = fmaf(sg, a.z, acc.z);
-          acc.w = fmaf(sg, a.w, acc.w);
-        }
-        float* out = SA + (long long)h * ldsa + col;
-        if (full && (ldsa % 4) == 0) {
-          *reinterpret_cast<float4*>(out) = acc;
-        } else {
-          out[0] = acc.x;
-          if (col + 1 < d) out[1] = acc.y;
-          if (col + 2 < d) out[2] = acc.z;
-          if (col + 3 < d) out[3] = acc.w;
-        }
-      }
-    }
-    __syncthreads();  // keys reused by the next bucket
   }
+  const int ct = threadIdx.x % CT, rg = threadIdx.x / CT;
+  const int col = 4 * (slice * CT + ct);
+  float4 acc = make_float4(0.f, 0.f, 0.f, 0.f);
+  if (col < d) {
+    const bool full = col + 4 <= d;
+    auto load = [&](int en) {
+      const float* row = A + (long long)entry_row(en) * lda + col;
+      if (full) return __ldcs(reinterpret_cast<const float4*>(row));
+      return make_float4(row[0], col + 1 < d ? row[1] : 0.f, col + 2 < d ? row[2] : 0.f, 0.f);
+    };
+    auto add = [&](int en, const float4& a) {
+      const float sg = entry_sign(en);
+      acc.x = fmaf(sg, a.x, acc.x);
+      acc.y = fmaf(sg, a.y, acc.y);
+      acc.z = fmaf(sg, a.z, acc.z);
+      acc.w = fmaf(sg, a.w, acc.w);
+    };
+    int e = rg;
+    for (; e + (kRowsInFlight - 1) * RG < cnt; e += kRowsInFlight * RG) {
+      int en[kRowsInFlight];
+      float4 a[kRowsInFlight];
+#pragma unroll
+      for (int u = 0; u < kRowsInFlight; ++u) en[u] = sorted ? keys[e + u * RG] : list[beg + e + u * RG];
+#pragma unroll
+      for (int u = 0; u < kRowsInFlight; ++u) a[u] = load(en[u]);
+#pragma unroll
+      for (int u = 0; u < kRowsInFlight; ++u) add(en[u], a[u]);
+    }
+    for (; e < cnt; e += RG) {
+      const int en = sorted ? keys[e] : list[beg + e];
+      add(en, load(en));
+    }
+  }
+  if constexpr (RG > 1) {
+    red[threadIdx.x] = acc;
+    __syncthreads();
+    if (rg != 0) return;
+#pragma unroll
+    for (int g = 1; g < RG; ++g) {
+      const float4 b = red[g * CT + ct];
+      acc.x += b.x;
+      acc.y += b.y;
+      acc.z += b.z;
+      acc.w += b.w;
+    }
+  }
+  if (col >= d) return;
+  float* o = out + ((long long)z * m + h) * ldo + col;
+  if (col + 4 <= d && vec_out) {
+    *reinterpret_cast<float4*>(o) = acc;
+  } else {
+    o[0] = acc.x;
+    if (col + 1 < d) o[1] = acc.y;
+    if (col + 2 < d) o[2] = acc.z;
+    if (col + 3 < d) o[3] = acc.w;
+  }
+}
+
+// SA[h][c] = Σ_z part[z][h][c] in order of z.
+__global__ void cs_reduce_kernel(const float* __restrict__ part, int ks, int m, int d, int dp, float* __restrict__ SA,
+                                 long long ldsa) {
+  const int c = blockIdx.x * blockDim.x + threadIdx.x, h = blockIdx.y;
+  if (c >= d) return;
+  float s = 0.f;
+  for (int z = 0; z < ks; ++z) s += part[((size_t)z * m + h) * dp + c];
+  SA[(long long)h * ldsa + c] = s;
 }
 
 }  // namespace
 
 int sketch_countsketch(const float* A, int64_t n, int64_t d, int64_t lda, int64_t m,
                        uint64_t seed, float* SA, int64_t ldsa, cudaStream_t s) {
+  const bool chunked = m <= kHistMaxM;
+  int64_t chunks = 1, rows = n;
+  if (chunked) {
+    chunks = (n + kChunkRows - 1) / kChunkRows;
+    if (chunks > kMaxChunks) chunks = kMaxChunks;
+    rows = round_up((n + chunks - 1) / chunks, 32);
+    chunks = (n + rows - 1) / rows;
+  }
+  // Column groups per block: the whole row up to 1024 columns (see the gather).
+  const int64_t groups = (d + 3) / 4;
+  int ct = 16;
+  while (ct < 256 && ct < groups) ct *= 2;
+  const int slices = (int)((groups + ct - 1) / ct);
+  // Chunk ranges per bucket: few and full buckets are cut so that two waves of
+  // blocks (8 per SM) share the work and a block's entries can be sorted, as
+  // long as a thread still has eight rows to keep in flight.
+  const int64_t units = m * slices;
+  const int64_t per_bucket = (n + m - 1) / m;
+  int64_t ks = (8LL * num_sms() + units - 1) / units;
+  const int64_t most = per_bucket / (kRowsInFlight * (kGatherThreads / ct));
+  if (ks > most) ks = most;
+  const int64_t need = (per_bucket + kSortCap / 2 - 1) / (kSortCap / 2);
+  if (ks < need) ks = need;
+  if (ks > chunks) ks = chunks;
+  if (ks < 1) ks = 1;
+
   StreamScratch scratch;
-  // code[n], list[n], counts[m], offsets[m+1], cursor[m]
-  const size_t bytes = sizeof(int) * ((size_t)2 * n + 3 * (size_t)m + 1);
+  const int64_t dp = round_up(d, 4);
+  // part[ks][m][dp] when ks > 1, code[n], list[n], hist/counts[chunks][m], start[chunks][m], cursor[m]
+  const size_t part_floats = ks > 1 ? (size_t)ks * m * dp : 0;
+  const size_t bytes = sizeof(float) * part_floats +
+                       sizeof(int) * ((size_t)2 * n + 2 * (size_t)chunks * m + (chunked ? 0 : (size_t)m));
   int rc = scratch.alloc(bytes, s);
   if (rc) return rc;
-  int* code = static_cast<int*>(scratch.p);
+  float* part = static_cast<float*>(scratch.p);
+  int* code = reinterpret_cast<int*>(part + part_floats);
   int* list = code + n;
-  int* counts = list + n;
-  int* offsets = counts + m;
-  int* cursor = offsets + m + 1;
-  MIHS_CUDA_TRY(cudaMemsetAsync(counts, 0, sizeof(int) * (size_t)m, s));
+  int* hist = list + n;
+  int* start = hist + (size_t)chunks * m;
   const uint32_t k0 = (uint32_t)seed, k1 = (uint32_t)(seed >> 32);
-  const int nb = (int)((n + 255) / 256);
-  cs_hash_kernel<<<nb, 256, 0, s>>>((int)n, (uint32_t)m, k0, k1, code, counts);
+  if (chunked) {
+    const size_t smem = sizeof(int) * (size_t)m;
+    cs_count_kernel<<<(unsigned)chunks, kSortThreads, smem, s>>>((int)n, (int)m, (int)rows, k0, k1, code, hist);
+    MIHS_CHECK_LAUNCH();
+    cs_scatter_kernel<<<(unsigned)chunks, kSortThreads, smem, s>>>((int)n, (int)m, (int)rows, code, hist, start, list);
+    MIHS_CHECK_LAUNCH();
+    count_launch(2);
+  } else {
+    int* cursor = start + m;
+    const int nb = (int)((n + 255) / 256);
+    MIHS_CUDA_TRY(cudaMemsetAsync(hist, 0, sizeof(int) * (size_t)m, s));
+    cs_hash_global_kernel<<<nb, 256, 0, s>>>((int)n, (uint32_t)m, k0, k1, code, hist);
+    MIHS_CHECK_LAUNCH();
+    cs_scan_kernel<<<1, 1024, 0, s>>>(hist, (int)m, start, cursor);
+    MIHS_CHECK_LAUNCH();
+    cs_scatter_global_kernel<<<nb, 256, 0, s>>>((int)n, code, cursor, list);
+    MIHS_CHECK_LAUNCH();
+    count_launch(3);
+  }
+  float* out = ks > 1 ? part : SA;
+  const long long ldo = ks > 1 ? (long long)dp : (long long)ldsa;
+  const int vec_out = ldo % 4 == 0 && (reinterpret_cast<uintptr_t>(out) & 15u) == 0;
+  const unsigned grid = (unsigned)(units * ks);
+  auto kern = ct == 256   ? cs_gather_kernel<256>
+              : ct == 128 ? cs_gather_kernel<128>
+              : ct == 64  ? cs_gather_kernel<64>
+              : ct == 32  ? cs_gather_kernel<32>
+                          : cs_gather_kernel<16>;
+  kern<<<grid, kGatherThreads, 0, s>>>(A, (int)n, (int)d, (long long)lda, start, list, (int)m, (int)chunks, (int)ks,
+                                       slices, out, ldo, vec_out);
   MIHS_CHECK_LAUNCH();
-  cs_scan_kernel<<<1, 1024, 0, s>>>(counts, (int)m, offsets, cursor);
-  MIHS_CHECK_LAUNCH();
-  cs_scatter_kernel<<<nb, 256, 0, s>>>((int)n, code, cursor, list);
-  MIHS_CHECK_LAUNCH();
-  const int grid = (int)(m < 65535 ? m : 65535);
-  cs_gather_kernel<<<grid, kGatherThreads, 0, s>>>(A, (int)d, (long long)lda, offsets, list,
-                                                    (int)m, SA, (long long)ldsa);
-  MIHS_CHECK_LAUNCH();
-  count_launch(4);
+  count_launch();
+  if (ks > 1) {
+    cs_reduce_kernel<<<dim3((unsigned)((d + 127) / 128), (unsigned)m), 128, 0, s>>>(part, (int)ks, (int)m, (int)d,
+                                                                                    (int)dp, SA, (long long)ldsa);
+    MIHS_CHECK_LAUNCH();
+    count_launch();
+  }
   return MIHS_OK;
 }
 
