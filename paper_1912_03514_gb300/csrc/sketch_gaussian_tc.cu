@@ -634,21 +634,6 @@ EncodeTiledFn encode_fn() {
 
 bool gaussian_tc_available() { return encode_fn() != nullptr; }
 
-int encode_tmap_2d_f32(CUtensorMap* map, const float* A, int64_t rows, int64_t cols, int64_t ld, int box_cols,
-                       int box_rows, int l2_promotion) {
-  EncodeTiledFn enc = encode_fn();
-  if (enc == nullptr) return MIHS_ERR_UNSUPPORTED;
-  const cuuint64_t gdim[2] = {(cuuint64_t)cols, (cuuint64_t)rows};
-  const cuuint64_t gstride[1] = {(cuuint64_t)ld * sizeof(float)};
-  const cuuint32_t box[2] = {(cuuint32_t)box_cols, (cuuint32_t)box_rows};
-  const cuuint32_t estr[2] = {1u, 1u};
-  const CUresult r = enc(map, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 2, const_cast<float*>(A), gdim, gstride, box, estr,
-                         CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_NONE,
-                         l2_promotion == 128 ? CU_TENSOR_MAP_L2_PROMOTION_L2_128B : CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
-                         CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
-  return r == CUDA_SUCCESS ? MIHS_OK : MIHS_ERR_UNSUPPORTED;
-}
-
 int sketch_gaussian_tc(const float* A, int64_t n, int64_t d, int64_t lda, int64_t m, uint64_t seed, float* SA,
                        int64_t ldsa, cudaStream_t s, int prec) {
   using KernFn = void (*)(const CUtensorMap, const GaussTcArgs);

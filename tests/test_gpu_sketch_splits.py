@@ -30,3 +30,21 @@ def test_countsketch_splits_are_exact(n, d, m):
     np.add.at(ref, h, A[:, :d].numpy().astype(np.float64) * np.asarray(sign, dtype=np.float64)[:, None])
     assert np.array_equal(SA.cpu().numpy().astype(np.float64), ref)
     assert np.array_equal(SA2.cpu().numpy().astype(np.float64), ref)
+
+
+# n, d, m: a single block of 1024 rows and one row more, fewer rows than a block, the last column pair alone, each
+# count of samples per thread and its first extra sample, more samples than one block of threads holds
+@pytest.mark.parametrize("n,d,m", [(1024, 16, 128), (1025, 17, 129), (3, 5, 2), (1, 1, 1), (2500, 31, 256),
+                                   (2500, 33, 257), (5000, 15, 385), (5000, 48, 513), (4100, 20, 640),
+                                   (4100, 20, 641), (9000, 3, 2000), (70001, 100, 64)])
+def test_srht_splits_are_exact(n, d, m):
+    """±1 sums of small integers are exact in fp32; only the factor 1/√m rounds, and the product with it."""
+    lda = (d + 3) // 4 * 4
+    A = torch.full((n, lda), float("nan"))
+    A[:, :d] = W.randint_matrix((n, d), n + d, -3, 3)
+    Ad = A.to(DEV).as_strided((n, d), (lda, 1))
+    out = torch.full((m, d + 1), float("nan"), device=DEV)[:, :d]  # rows of SA not 16-byte aligned
+    SA = mihs.sketch_apply(Ad, o.SRHT, m, 5 + m, SA=out).cpu().numpy().astype(np.float64)
+    ref = o.sketch_apply(o.SRHT, A[:, :d].numpy().astype(np.float64), m, 5 + m)
+    sums = np.rint(ref * np.sqrt(m))  # the integers themselves (the oracle's own fp64 rounding dropped)
+    assert np.all(np.abs(SA * np.sqrt(m) - sums) <= 2.0 ** -22 * np.abs(sums))
