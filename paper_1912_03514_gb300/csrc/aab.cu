@@ -17,7 +17,11 @@
 //     from partials summed in a fixed order, so all blocks take the same
 //     branch and the result is deterministic.
 // The d-vectors of the recursion (v, d, x) are replicated per block (O(d)
-// work, negligible next to the O(md/CL) products).  When SA is too large for
+// work, negligible next to the O(md/CL) products).
+//
+// That is the form for sketches whose rows fit the shared memory of a cluster
+// but not its registers; aab_reg.cu, which is faster (78 against 141 µs for 30
+// passes at 588 × 1024), takes all that do.  When SA is too large for
 // the shared memory of 16 blocks, launch_aab hands a single-λ solve that has
 // scratch to the grid form (aab_grid.cu); otherwise the cluster's blocks
 // read their rows of SA from global memory (L2) on every pass.
@@ -47,7 +51,19 @@ struct ClusterPlan {
   int cl;
   int in_smem;
   size_t smem;
+  int reg_rows;  // rows per warp of the register form; 0: the shared-memory (or L2) form
+  int cols_per, cols_log2;  // column slice per block
 };
+
+// Column slice of a block: a power of two ≥ 4 that cl blocks cover dp with.
+void plan_columns(ClusterPlan& p, int dp) {
+  p.cols_per = 4;
+  p.cols_log2 = 2;
+  while ((int64_t)p.cols_per * p.cl < dp) {
+    p.cols_per <<= 1;
+    ++p.cols_log2;
+  }
+}
 
 size_t elem_bytes(int sa_type) { return sa_type == MIHS_SA_BF16 ? 2 : (sa_type == MIHS_SA_FP8E4M3 ? 1 : 4); }
 
@@ -63,7 +79,8 @@ size_t smem_bytes(int m, int dp, int cl, bool in_smem, int sa_type) {
   return base;
 }
 
-bool cluster_fits(int cl, int dp, size_t smem, int sa_type) {
+// Whether a cluster of cl blocks of the kernel can be resident.
+bool cluster_fits(int cl, const void* fn, size_t smem) {
   cudaLaunchConfig_t cfg = {};
   cudaLaunchAttribute attr[1];
   attr[0].id = cudaLaunchAttributeClusterDimension;
@@ -76,7 +93,7 @@ bool cluster_fits(int cl, int dp, size_t smem, int sa_type) {
   cfg.attrs = attr;
   cfg.numAttrs = 1;
   int nclusters = 0;
-  if (cudaOccupancyMaxActiveClusters(&nclusters, (void*)kernel_for(cl, dp, sa_type), &cfg) != cudaSuccess) {
+  if (cudaOccupancyMaxActiveClusters(&nclusters, fn, &cfg) != cudaSuccess) {
     cudaGetLastError();
     return false;
   }
@@ -98,12 +115,32 @@ ClusterPlan plan_cluster_uncached(int m, int dp, int sa_type) {
   int forced = 0;
   if (const char* e = std::getenv("MIHS_AAB_CLUSTER")) forced = std::atoi(e);
   const int sizes[] = {1, 2, 4, 8, 16};
+  // Smallest cluster whose registers hold SA.
+  for (int cl : sizes) {
+    if (forced > 0 && cl != forced) continue;
+    if (cl > m && cl > 1) break;
+    const int r = aab_reg_rows(m, cl, dp);
+    if (r == 0) continue;
+    ClusterPlan p = {cl, 1, 0, r, 0, 0};
+    plan_columns(p, dp);
+    p.smem = aab_reg_smem(dp, cl, p.cols_per);
+    const void* fn = aab_reg_fn(dp, r);
+    if (cudaFuncSetAttribute(fn, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) == cudaSuccess &&
+        cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmemBudget) == cudaSuccess &&
+        cluster_fits(cl, fn, p.smem))
+      return p;
+    cudaGetLastError();
+  }
   // Smallest cluster whose row slices of SA fit in shared memory.
   for (int cl : sizes) {
     if (forced > 0 && cl != forced) continue;
     if (cl > m && cl > 1) break;
     const size_t sm = smem_bytes(m, dp, cl, true, sa_type);
-    if (sm <= kSmemBudget && cluster_fits(cl, dp, sm, sa_type)) return {cl, 1, sm};
+    if (sm <= kSmemBudget && cluster_fits(cl, (const void*)kernel_for(cl, dp, sa_type), sm)) {
+      ClusterPlan p = {cl, 1, sm, 0, 0, 0};
+      plan_columns(p, dp);
+      return p;
+    }
   }
   // Otherwise the largest launchable cluster reading SA from global memory (L2).
   for (int i = 4; i >= 0; --i) {
@@ -111,9 +148,13 @@ ClusterPlan plan_cluster_uncached(int m, int dp, int sa_type) {
     if (forced > 0 && cl != forced) continue;
     if (cl > m && cl > 1) continue;
     const size_t sm = smem_bytes(m, dp, cl, false, sa_type);
-    if (sm <= kSmemBudget && cluster_fits(cl, dp, sm, sa_type)) return {cl, 0, sm};
+    if (sm <= kSmemBudget && cluster_fits(cl, (const void*)kernel_for(cl, dp, sa_type), sm)) {
+      ClusterPlan p = {cl, 0, sm, 0, 0, 0};
+      plan_columns(p, dp);
+      return p;
+    }
   }
-  return {0, 0, 0};
+  return {0, 0, 0, 0, 0, 0};
 }
 
 std::mutex g_plan_mu;
@@ -197,12 +238,8 @@ int launch_aab(const AabLaunch& a, cudaStream_t s) {
   }
   P.rpc = (a.m + cp.cl - 1) / cp.cl;
   P.rpc_pad = (int)round_up(P.rpc, 4);
-  {
-    int cp2 = 4, lg = 2;
-    while ((int64_t)cp2 * cp.cl < P.dp) { cp2 <<= 1; ++lg; }
-    P.cols_per = cp2;
-    P.cols_log2 = lg;
-  }
+  P.cols_per = cp.cols_per;
+  P.cols_log2 = cp.cols_log2;
   P.sa_in_smem = cp.in_smem;
   P.sa_pitch = smem_pitch(P.dp, a.sa_type);
   P.sa_vec = (a.ldsa % 4 == 0 && (reinterpret_cast<uintptr_t>(a.SA) & 15u) == 0) ? 1 : 0;
@@ -225,7 +262,13 @@ int launch_aab(const AabLaunch& a, cudaStream_t s) {
   cfg.attrs = attr;
   cfg.numAttrs = 1;
   timing_begin(kTimerAab, s);
-  MIHS_CUDA_TRY(cudaLaunchKernelEx(&cfg, kernel_for(cp.cl, P.dp, a.sa_type), P));
+  if (cp.reg_rows > 0) {
+    int sa_type = a.sa_type, cl = cp.cl;
+    void* args[] = {&P, &sa_type, &cl};
+    MIHS_CUDA_TRY(cudaLaunchKernelExC(&cfg, aab_reg_fn(P.dp, cp.reg_rows), args));
+  } else {
+    MIHS_CUDA_TRY(cudaLaunchKernelEx(&cfg, kernel_for(cp.cl, P.dp, a.sa_type), P));
+  }
   timing_end(kTimerAab, s);
   count_launch();
   return MIHS_OK;

@@ -525,7 +525,10 @@ int mihs_device_status(int* code) {
   int gr = 0;
   rc = aab_grid_device_error(&gr);
   if (rc) return rc;
-  *code = a ? a : (g ? g : (dd ? dd : (pa ? pa : (ab ? ab : gr))));
+  int re = 0;
+  rc = aab_reg_device_error(&re);
+  if (rc) return rc;
+  *code = a ? a : (g ? g : (dd ? dd : (pa ? pa : (ab ? ab : (gr ? gr : re)))));
   return MIHS_OK;
 }
 

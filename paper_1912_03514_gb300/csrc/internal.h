@@ -138,6 +138,7 @@ constexpr size_t kAabGridBarBytes = 256;
 size_t aab_grid_ws_bytes(int d);
 int launch_aab_grid(const AabLaunch& a, void* ws, cudaStream_t s);
 int aab_grid_device_error(int* code);
+int aab_reg_device_error(int* code);
 // True when launch_aab would take the grid form given scratch: `form` is
 // MIHS_AAB_GRID, or MIHS_AAB_AUTO and SA of m × d does not fit in the shared
 // memory of one cluster (for AUTO, MIHS_AAB_FORM=grid or =cluster in the
