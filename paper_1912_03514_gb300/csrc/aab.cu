@@ -20,7 +20,7 @@
 // work, negligible next to the O(md/CL) products).
 //
 // That is the form for sketches whose rows fit the shared memory of a cluster
-// but not its registers; aab_reg.cu, which is faster (78 against 141 µs for 30
+// but not its registers; aab_reg.cuh, which is faster (66 against 141 µs for 30
 // passes at 588 × 1024), takes all that do.  When SA is too large for
 // the shared memory of 16 blocks, launch_aab hands a single-λ solve that has
 // scratch to the grid form (aab_grid.cu); otherwise the cluster's blocks
@@ -47,11 +47,21 @@ AabKernelFn kernel_for(int cl, int dp, int sa_type) {
   return kernel_for_f32(cl, dp);
 }
 
+RegKernel reg_kernel(int cl, int m, int dp) {
+  switch (cl) {
+    case 1: return reg_kernel_1(m, dp);
+    case 2: return reg_kernel_2(m, dp);
+    case 4: return reg_kernel_4(m, dp);
+    case 8: return reg_kernel_8(m, dp);
+    default: return reg_kernel_16(m, dp);
+  }
+}
+
 struct ClusterPlan {
   int cl;
   int in_smem;
   size_t smem;
-  int reg_rows;  // rows per warp of the register form; 0: the shared-memory (or L2) form
+  const void* reg_fn;  // kernel of the register form; null: the shared-memory (or L2) form
   int cols_per, cols_log2;  // column slice per block
 };
 
@@ -119,16 +129,12 @@ ClusterPlan plan_cluster_uncached(int m, int dp, int sa_type) {
   for (int cl : sizes) {
     if (forced > 0 && cl != forced) continue;
     if (cl > m && cl > 1) break;
-    const int r = aab_reg_rows(m, cl, dp);
-    if (r == 0) continue;
-    ClusterPlan p = {cl, 1, 0, r, 0, 0};
-    plan_columns(p, dp);
-    p.smem = aab_reg_smem(dp, cl, p.cols_per);
-    const void* fn = aab_reg_fn(dp, r);
-    if (cudaFuncSetAttribute(fn, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) == cudaSuccess &&
-        cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmemBudget) == cudaSuccess &&
-        cluster_fits(cl, fn, p.smem))
-      return p;
+    const RegKernel rk = reg_kernel(cl, m, dp);
+    if (rk.fn == nullptr) continue;
+    if (cudaFuncSetAttribute(rk.fn, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) == cudaSuccess &&
+        cudaFuncSetAttribute(rk.fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)rk.smem) == cudaSuccess &&
+        cluster_fits(cl, rk.fn, rk.smem))
+      return {cl, 1, rk.smem, rk.fn, 0, 0};
     cudaGetLastError();
   }
   // Smallest cluster whose row slices of SA fit in shared memory.
@@ -137,7 +143,7 @@ ClusterPlan plan_cluster_uncached(int m, int dp, int sa_type) {
     if (cl > m && cl > 1) break;
     const size_t sm = smem_bytes(m, dp, cl, true, sa_type);
     if (sm <= kSmemBudget && cluster_fits(cl, (const void*)kernel_for(cl, dp, sa_type), sm)) {
-      ClusterPlan p = {cl, 1, sm, 0, 0, 0};
+      ClusterPlan p = {cl, 1, sm, nullptr, 0, 0};
       plan_columns(p, dp);
       return p;
     }
@@ -149,12 +155,12 @@ ClusterPlan plan_cluster_uncached(int m, int dp, int sa_type) {
     if (cl > m && cl > 1) continue;
     const size_t sm = smem_bytes(m, dp, cl, false, sa_type);
     if (sm <= kSmemBudget && cluster_fits(cl, (const void*)kernel_for(cl, dp, sa_type), sm)) {
-      ClusterPlan p = {cl, 0, sm, 0, 0, 0};
+      ClusterPlan p = {cl, 0, sm, nullptr, 0, 0};
       plan_columns(p, dp);
       return p;
     }
   }
-  return {0, 0, 0, 0, 0, 0};
+  return {0, 0, 0, nullptr, 0, 0};
 }
 
 std::mutex g_plan_mu;
@@ -170,6 +176,18 @@ ClusterPlan plan_cluster(int m, int dp, int sa_type) {
 }
 
 }  // namespace
+
+int aab_reg_device_error(int* code) {
+  int (*const words[])(int*) = {reg_error_1, reg_error_2, reg_error_4, reg_error_8, reg_error_16};
+  *code = 0;
+  for (auto word : words) {
+    int v = 0;
+    const int rc = word(&v);
+    if (rc) return rc;
+    if (*code == 0) *code = v;
+  }
+  return MIHS_OK;
+}
 
 void aab_prepare(int m, int d, int sa_type) { (void)plan_cluster(m, (int)round_up(d, 4), sa_type); }
 
@@ -262,10 +280,10 @@ int launch_aab(const AabLaunch& a, cudaStream_t s) {
   cfg.attrs = attr;
   cfg.numAttrs = 1;
   timing_begin(kTimerAab, s);
-  if (cp.reg_rows > 0) {
-    int sa_type = a.sa_type, cl = cp.cl;
-    void* args[] = {&P, &sa_type, &cl};
-    MIHS_CUDA_TRY(cudaLaunchKernelExC(&cfg, aab_reg_fn(P.dp, cp.reg_rows), args));
+  if (cp.reg_fn != nullptr) {
+    int sa_type = a.sa_type;
+    void* args[] = {&P, &sa_type};
+    MIHS_CUDA_TRY(cudaLaunchKernelExC(&cfg, cp.reg_fn, args));
   } else {
     MIHS_CUDA_TRY(cudaLaunchKernelEx(&cfg, kernel_for(cp.cl, P.dp, a.sa_type), P));
   }

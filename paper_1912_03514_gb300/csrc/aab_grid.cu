@@ -480,20 +480,25 @@ struct GridPlan {
   size_t smem = 0;
 };
 
-// Rows per block so that SA is spread over `blocks` blocks (0: one per SM),
-// raised to the fewest blocks whose row slices fit in shared memory, and the
-// launch that holds it; G = 0 when SA does not fit even one block per SM.
-GridPlan plan_grid(int m, int dp, int sa_type, int blocks) {
-  GridPlan gp;
-  const int nsm = num_sms();
-  int want = nsm;
+// Blocks asked for by the caller, or by the environment when it did not ask; one per SM otherwise.
+int grid_blocks_wanted(int blocks) {
+  int want = num_sms();
   if (blocks > 0) {
     want = blocks;
   } else if (const char* e = std::getenv("MIHS_AAB_GRID_BLOCKS")) {
     const int v = std::atoi(e);
     if (v > 0) want = v;
   }
-  if (want > nsm) want = nsm;
+  return want < num_sms() ? want : num_sms();
+}
+
+// Rows per block so that SA is spread over `blocks` blocks (0: one per SM),
+// raised to the fewest blocks whose row slices fit in shared memory, and the
+// launch that holds it; G = 0 when SA does not fit even one block per SM.
+GridPlan plan_grid(int m, int dp, int sa_type, int blocks) {
+  GridPlan gp;
+  const int nsm = num_sms();
+  int want = grid_blocks_wanted(blocks);
   const int pitch = sa_type == MIHS_SA_FP32 ? dp : (int)round_up(dp, 16);
   for (;; want = std::min(nsm, want + (want < 8 ? 1 : want / 8))) {
     const int R = (m + want - 1) / want;
@@ -522,7 +527,13 @@ std::mutex g_grid_mu;
 size_t aab_grid_ws_bytes(int d) {
   const size_t dp = (size_t)round_up(d, 4);
   const size_t G4 = (size_t)round_up(num_sms(), 4);
-  return kAabGridBarBytes + sizeof(float) * (G4 * dp + 2 * G4 + dp);
+  return kAabGridBarBytes + (size_t)round_up((int64_t)aab_gridreg_ws_bytes(d), 256) +
+         sizeof(float) * (G4 * dp + 2 * G4 + dp);
+}
+
+int aab_grid_ws_init(void* ws, int d, cudaStream_t s) {
+  MIHS_CUDA_TRY(cudaMemsetAsync(ws, 0, kAabGridBarBytes + aab_gridreg_ws_bytes(d), s));
+  return MIHS_OK;
 }
 
 int aab_grid_device_error(int* code) {
@@ -541,6 +552,12 @@ int launch_aab_grid(const AabLaunch& a, void* ws, cudaStream_t s) {
   const bool vec = (reinterpret_cast<uintptr_t>(a.SA) & 15u) == 0 &&
                    (a.sa_type != MIHS_SA_FP32 || a.ldsa % 4 == 0);
   if (a.sa_type != MIHS_SA_FP32 && (!vec || a.ldsa < round_up(dp, 16))) return MIHS_ERR_UNSUPPORTED;
+  // In registers where the blocks asked for hold SA there (30 passes at
+  // 3076 × 2048: 144 against 228 µs), else in shared memory.
+  {
+    const int rc = launch_aab_gridreg(a, grid_blocks_wanted(a.grid_blocks), static_cast<char*>(ws) + kAabGridBarBytes, s);
+    if (rc != MIHS_ERR_UNSUPPORTED) return rc;
+  }
   const GridPlan gp = plan_grid(a.m, dp, a.sa_type, a.grid_blocks);
   if (gp.G == 0) return MIHS_ERR_UNSUPPORTED;
   const GridFn fn = grid_kernel(dp, a.sa_type);
@@ -584,7 +601,8 @@ int launch_aab_grid(const AabLaunch& a, void* ws, cudaStream_t s) {
   P.cond = a.cond;
   const size_t G4 = (size_t)round_up(num_sms(), 4);
   P.bar = static_cast<unsigned int*>(ws);
-  float* f = reinterpret_cast<float*>(static_cast<char*>(ws) + kAabGridBarBytes);
+  float* f = reinterpret_cast<float*>(static_cast<char*>(ws) + kAabGridBarBytes +
+                                      round_up((int64_t)aab_gridreg_ws_bytes(a.d), 256));
   P.Upart = f;
   P.rho2 = f + G4 * dp;
   P.theta2 = P.rho2 + G4;

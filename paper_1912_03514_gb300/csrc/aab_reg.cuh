@@ -17,26 +17,33 @@
 //     barrier and no remote load;
 //   * one block barrier per pass (the eight warps' shares of u);
 //   * scalars off the chain: v is sent before the rotation, the φ recursion
-//     and the forward substitution are computed, and the dots start on θv
-//     before θ is known.
-// 588 × 1024, 30 passes: 141 → 78 µs (2.4 µs per pass; the form with SA in
-// shared memory swept it twice per pass and crossed two cluster barriers and
-// two remote-load round trips, 4.6 µs).
+//     and the forward substitution are computed; the dots start on θv before θ
+//     is known, and θ² is one more of them, taken by every warp from the whole
+//     vector rather than exchanged.
+// 588 × 1024, 30 passes: 141 → 66 µs, 700 × 256: 177 → 50 µs (the form with SA
+// in shared memory swept it twice per pass and crossed two cluster barriers
+// and two remote-load round trips).
 // Every sum has a fixed order and every block computes the same scalars from
 // the same numbers, so all blocks take the same branches.  Quantised SA is
 // decoded once, into fp32 registers.
 //
-// Buffers are reused from pass to pass without further barriers: a block
-// sends its share of u(k + 1) only after all of v(k + 1) has arrived, v(k + 1)
-// only after all of u(k); so by the time a buffer is written again everyone
-// who had to read it has sent something that depends on it.  (The ρ² slots
-// are read by warps that send nothing in between: they alternate.)
+// Buffers are reused from pass to pass without further barriers.  θv: a block
+// sends its share of u(k + 1) once all its warps have read θv(k) (the block
+// barrier of its sweep), and θv(k + 1) goes out only when all shares of
+// u(k + 1) have come.  Shares of u and ρ² alternate between two buffers: a
+// block may receive those of pass k + 1 while some of its own warps still read
+// those of pass k (a peer waits for one copy of the slice's warps, not for
+// all), but those of pass k + 2 only after its own share of u(k + 1), which
+// all its warps have reached the sweep's barrier for.
+#pragma once
+
 #include "aab_kernel.cuh"
 
 namespace mihs {
 namespace aabk {
 namespace {
 
+// One error word per translation unit (each instantiates one cluster size).
 __device__ int g_aab_reg_error = 0;
 
 __device__ __forceinline__ uint32_t mapa_u32(uint32_t saddr, uint32_t rank) {
@@ -98,43 +105,63 @@ __device__ __forceinline__ float2 p2_unpack(P2 v) {
   return r;
 }
 
-// Shared memory of a block (floats; every region a multiple of 4).
-struct RegSmem {
-  int z, ubuf, wpart, rbuf, tbuf, red, bars, total;
+// The shape of a cluster: CL blocks, CH chunks of 128 columns (narrower SA is
+// zero-padded), all of it known at compile time: a pass has ≈ 550 instructions
+// per warp and two warps per scheduler, so every index computed at run time
+// lengthens the chain (≈ 6 cycles per instruction; with run-time cluster and
+// slice sizes 588 × 1024 took 93 µs).
+template <int CL, int CH>
+struct RegShape {
+  static constexpr int DP = 128 * CH;
+  static constexpr int COLS = DP / CL;              // columns of a block's slice
+  static constexpr int NGS = COLS / 4;              // groups of four in it
+  static constexpr int NG = DP / 4 > kThreads ? DP / 4 / kThreads : 1;   // groups per thread, all columns
+  static constexpr int NQ = NGS > kThreads ? NGS / kThreads : 1;         // groups per thread of the slice
+  static constexpr int NW = NGS > 32 ? (NGS < kThreads ? NGS / 32 : kWarps) : 1;  // warps that the slice fills
+  static constexpr int H = NGS < 32 ? 32 / NGS : 1; // lanes per group of a narrow slice: each sums some ranks
+  static constexpr int REPS = kWarps / NW < 4 ? kWarps / NW : 4;  // copies of those warps: each sends to some ranks
+  static constexpr int RPL = CL > H ? CL / H : 1;   // ranks summed per lane
+  static constexpr int SPL = CL > H * REPS ? CL / (H * REPS) : 1;  // ranks sent to per lane
+  // shared memory (floats; every region a multiple of 4)
+  static constexpr int z = 0;                       // DP: θv, all columns (written by the owners)
+  static constexpr int ubuf = z + DP;               // 2 × CL × COLS: the blocks' shares of u on the own slice
+  static constexpr int wpart = ubuf + 2 * DP;       // kWarps × DP: the warps' shares of u
+  static constexpr int rbuf = wpart + kWarps * DP;  // 2 × 16: the blocks' shares of ρ²
+  static constexpr int red = rbuf + 32;             // kWarps
+  static constexpr int bars = red + kWarps;         // two mbarriers
+  static constexpr size_t bytes = sizeof(float) * (bars + 4);
 };
-__host__ __device__ inline RegSmem reg_smem(int dp, int cl, int cols_per) {
-  RegSmem L;
-  L.z = 0;                            // dp: θv, all columns (written by the owners)
-  L.ubuf = L.z + dp;                  // cl × cols_per: the blocks' shares of u on the own slice
-  L.wpart = L.ubuf + cl * cols_per;   // kWarps × dp: the warps' shares of u
-  L.rbuf = L.wpart + kWarps * dp;     // 2 × 16: the blocks' shares of ρ²
-  L.tbuf = L.rbuf + 32;               // 16: shares of θ² (one per block and slice warp)
-  L.red = L.tbuf + 16;                // kWarps + staging
-  L.bars = L.red + kWarps;            // two mbarriers
-  L.total = L.bars + 4;
-  return L;
+
+// Σ of N ≤ 16 values in a fixed order (a broadcast read).
+template <int N>
+__device__ __forceinline__ float sum_n(const float* p) {
+  if constexpr (N < 4) {
+    float s = p[0];
+#pragma unroll
+    for (int i = 1; i < N; ++i) s += p[i];
+    return s;
+  } else {
+    float s = 0.f;
+#pragma unroll
+    for (int i = 0; i < N; i += 4) {
+      const float4 a = *reinterpret_cast<const float4*>(p + i);
+      s += (a.x + a.y) + (a.z + a.w);
+    }
+    return s;
+  }
 }
 
-// Σ of up to 16 values in a fixed order (a broadcast read; values past `cnt` are zero).
-__device__ __forceinline__ float sum16(const float* p, int cnt) {
-  const float4* q = reinterpret_cast<const float4*>(p);
-  float4 a = q[0];
-  float s = (a.x + a.y) + (a.z + a.w);
-  if (cnt > 4) {
-    const float4 b = q[1];
-    s += (b.x + b.y) + (b.z + b.w);
-  }
-  if (cnt > 8) {
-    const float4 c = q[2], e = q[3];
-    s += ((c.x + c.y) + (c.z + c.w)) + ((e.x + e.y) + (e.z + e.w));
-  }
-  return s;
+__device__ __forceinline__ P2 p2_add(P2 a, P2 b) {
+  P2 d;
+  asm("add.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
+  return d;
 }
 
-// CH: chunks of 128 columns; R: rows per warp (R·CH·4 ≤ 160 registers).
-template <int CH, int R>
-__global__ void __launch_bounds__(kThreads, 1) aab_reg_kernel(const AabParams P, int sa_type, int cl) {
-  constexpr int NG = CH > 8 ? 2 : 1;  // column groups (16 bytes) per thread: dp/4 ≤ 256·NG
+// R: rows per warp (R·CH·4 ≤ 160 registers).
+template <int CL, int CH, int R>
+__global__ void __launch_bounds__(kThreads, 1) aab_reg_kernel(const AabParams P, int sa_type) {
+  using S = RegShape<CL, CH>;
+  constexpr int DP = S::DP, NG = S::NG, NQ = S::NQ;
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   uint32_t rank;
   asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(rank));
@@ -153,14 +180,12 @@ __global__ void __launch_bounds__(kThreads, 1) aab_reg_kernel(const AabParams P,
 
   extern __shared__ float4 smem4[];
   float* sm = reinterpret_cast<float*>(smem4);
-  const RegSmem L = reg_smem(dp, cl, P.cols_per);
-  float* z = sm + L.z;
-  float* ubuf = sm + L.ubuf;
-  float* wpart = sm + L.wpart;
-  float* rbuf = sm + L.rbuf;
-  float* tbuf = sm + L.tbuf;
-  float* red = sm + L.red;
-  uint64_t* barA = reinterpret_cast<uint64_t*>(sm + L.bars);
+  float* z = sm + S::z;
+  float* ubuf = sm + S::ubuf;
+  float* wpart = sm + S::wpart;
+  float* rbuf = sm + S::rbuf;
+  float* red = sm + S::red;
+  uint64_t* barA = reinterpret_cast<uint64_t*>(sm + S::bars);
   uint64_t* barB = barA + 1;
 
   // Solve-mode control block: every block reads it before the cluster
@@ -179,20 +204,11 @@ __global__ void __launch_bounds__(kThreads, 1) aab_reg_kernel(const AabParams P,
     refresh = ctl_->refresh;
     corr = ctl_->corr;
   }
-  // Column slice of this block: groups (4 columns) [G0, G0 + ng), the first
-  // ngr of which lie below dp.  ng is a power of two; with fewer than 32
-  // groups the lanes of warp 0 share them, H lanes per group.
-  const int ng = P.cols_per >> 2;
-  const int G0 = (int)rank * ng, groups = dp >> 2;
-  const int ngr = max(0, min(groups - G0, ng));
-  const int nw = max(1, min(kWarps, ng >> 5));  // warps that own groups
-  const int H = ng < 32 ? 32 / ng : 1;
   if (tid == 0) {
     mbar_init(barA, 1);
     mbar_init(barB, 1);
     fence_mbar_init();
   }
-  if (tid < 48) rbuf[tid] = 0.f;  // rbuf and tbuf: slots past the cluster's stay zero
   __syncthreads();
   cluster_arrive();
   if (done) {
@@ -229,7 +245,7 @@ __global__ void __launch_bounds__(kThreads, 1) aab_reg_kernel(const AabParams P,
     }
   }
   float gsq = 0.f;
-  for (int j = tid; j < dp; j += kThreads) {
+  for (int j = tid; j < DP; j += kThreads) {
     const float gj = j < d ? g_in[j] : 0.f;
     z[j] = gj;
     gsq = fmaf(gj, gj, gsq);
@@ -270,33 +286,35 @@ __global__ void __launch_bounds__(kThreads, 1) aab_reg_kernel(const AabParams P,
   }
 
   // Bytes that arrive here per exchange: the blocks' u on the own slice and
-  // their ρ² shares; all of θv and the slice warps' θ² shares.
-  const uint32_t bytesA = (uint32_t)cl * (16u * (uint32_t)ngr + 4u);
-  const uint32_t bytesB = 16u * (uint32_t)groups + 4u * (uint32_t)(cl * nw);
+  // their ρ² shares; all of θv.
+  constexpr uint32_t bytesA = CL * (16u * S::NGS + 4u), bytesB = 4u * DP;
   const uint32_t a_barA = smem_u32(barA), a_barB = smem_u32(barB);
-  const uint32_t a_z = smem_u32(z), a_tbuf = smem_u32(tbuf);
   // Where this thread's column group(s) of u go: owner block and place there.
   uint32_t u_dst[NG], u_bar[NG];
 #pragma unroll
   for (int q = 0; q < NG; ++q) {
-    const int gq = tid + kThreads * q;
-    const uint32_t own = (uint32_t)((4 * gq) >> P.cols_log2);
-    const uint32_t o = own < (uint32_t)cl ? own : 0u;
-    u_dst[q] = mapa_u32(smem_u32(ubuf) + 4u * (rank * (uint32_t)P.cols_per + (uint32_t)(4 * gq - (int)o * P.cols_per)), o);
+    const int gq = min(tid + kThreads * q, DP / 4 - 1);
+    const uint32_t o = (uint32_t)(gq / S::NGS);
+    u_dst[q] = mapa_u32(smem_u32(ubuf) + 16u * (rank * (uint32_t)S::NGS + (uint32_t)(gq % S::NGS)), o);
     u_bar[q] = mapa_u32(a_barA, o);
   }
-  // Slice ownership of this thread: group(s) gsl + 256·q with ranks
-  // [h·cl/H …) summed by lane share h (H > 1: warp 0 only).
-  const int gsl = H > 1 ? (lane & (ng - 1)) : tid;
-  const int hsh = H > 1 ? lane / ng : 0;
-  const bool slice_warp = H > 1 ? warp == 0 : warp < nw;
-  const int hr0 = hsh * cl / H, hr1 = (hsh + 1) * cl / H;  // ranks this lane sums and sends to
-  float4 zo[NG], dv[NG], xs[NG];  // own slice: θv, d, x
+  const uint32_t r_dst = mapa_u32(smem_u32(rbuf) + 4u * rank, (uint32_t)(lane % CL));
+  const uint32_t r_bar = mapa_u32(a_barA, (uint32_t)(lane % CL));
+  // Slice ownership of this thread: group(s) gsl + 256·q.  The H lanes of a
+  // group sum the shares of RPL ranks each; every copy of the slice's warps
+  // does, and lane share `sh` of the H·REPS sends to SPL ranks.
+  const int rep = warp / S::NW;
+  const int gsl = S::H > 1 ? lane % S::NGS : (warp % S::NW) * 32 + lane;
+  const int hsh = S::H > 1 ? lane / S::NGS : 0, sh = rep * S::H + hsh;
+  const bool slice_warp = rep < S::REPS;
+  const bool sums = S::H <= CL || hsh < CL, sends = sh * S::SPL < CL;
+  const float* u_src = ubuf + (size_t)(hsh * S::RPL) * S::COLS + 4 * gsl;
+  const uint32_t z_src = smem_u32(z) + 4u * rank * S::COLS + 16u * (uint32_t)gsl;
+  float4 zo[NQ], dv[NQ], xs[NQ];  // own slice: θv, d, x
 #pragma unroll
-  for (int q = 0; q < NG; ++q) {
-    zo[q] = make_float4(0.f, 0.f, 0.f, 0.f);
-    dv[q] = xs[q] = zo[q];
-    if (slice_warp && gsl + kThreads * q < ngr) zo[q] = *reinterpret_cast<const float4*>(z + 4 * (G0 + gsl + kThreads * q));
+  for (int q = 0; q < NQ; ++q) {
+    zo[q] = *reinterpret_cast<const float4*>(z + rank * S::COLS + 4 * (gsl + kThreads * q));
+    dv[q] = xs[q] = make_float4(0.f, 0.f, 0.f, 0.f);
   }
 
   int k = 0;
@@ -315,29 +333,35 @@ __global__ void __launch_bounds__(kThreads, 1) aab_reg_kernel(const AabParams P,
     for (uint32_t it = 0;; ++it) {
       const uint32_t par = it & 1u;
       // ---- sweep: w = SA·v − θp with v = z/θ, this warp's rows
-      P2 s2[R];
+      P2 s2[R + 1];  // the rows' dots, and ‖z‖² = θ²
 #pragma unroll
-      for (int r = 0; r < R; ++r) s2[r] = 0ull;
+      for (int r = 0; r <= R; ++r) s2[r] = 0ull;
 #pragma unroll
       for (int ch = 0; ch < CH; ++ch) {
         const int j = 4 * lane + 128 * ch;
-        const ulonglong2 zz = *reinterpret_cast<const ulonglong2*>(z + (j < dp ? j : 0));  // SA is zero past dp
+        const ulonglong2 zz = *reinterpret_cast<const ulonglong2*>(z + j);
 #pragma unroll
         for (int r = 0; r < R; ++r) {
           s2[r] = p2_fma(sa[r][ch][0], zz.x, s2[r]);
           s2[r] = p2_fma(sa[r][ch][1], zz.y, s2[r]);
         }
+        s2[R] = p2_fma(zz.x, zz.x, s2[R]);
+        s2[R] = p2_fma(zz.y, zz.y, s2[R]);
       }
-      float w[R];
+      float w[R + 1];
 #pragma unroll
-      for (int r = 0; r < R; ++r) {
+      for (int r = 0; r <= R; ++r) {
         const float2 f = p2_unpack(s2[r]);
         w[r] = f.x + f.y;
       }
 #pragma unroll
       for (int o = 16; o > 0; o >>= 1) {
 #pragma unroll
-        for (int r = 0; r < R; ++r) w[r] += __shfl_xor_sync(0xffffffffu, w[r], o);
+        for (int r = 0; r <= R; ++r) w[r] += __shfl_xor_sync(0xffffffffu, w[r], o);
+      }
+      if (it > 0) {  // θ from the whole vector, the same in every warp of every block
+        norm_of(w[R], theta, inv_theta);
+        if (!(theta > 0.f)) break;  // invariant subspace
       }
       float rsq = 0.f;
 #pragma unroll
@@ -346,7 +370,7 @@ __global__ void __launch_bounds__(kThreads, 1) aab_reg_kernel(const AabParams P,
         rsq = fmaf(w[r], w[r], rsq);
       }
       // ---- u = Σ w_i·SA_i, chunk by chunk into the warp's share
-      float* wp = wpart + (size_t)warp * dp;
+      float* wp = wpart + warp * DP;
 #pragma unroll
       for (int ch = 0; ch < CH; ++ch) {
         const int j = 4 * lane + 128 * ch;
@@ -357,7 +381,7 @@ __global__ void __launch_bounds__(kThreads, 1) aab_reg_kernel(const AabParams P,
           u0 = p2_fma(sa[r][ch][0], wr, u0);
           u1 = p2_fma(sa[r][ch][1], wr, u1);
         }
-        if (j < dp) *reinterpret_cast<ulonglong2*>(wp + j) = make_ulonglong2(u0, u1);
+        *reinterpret_cast<ulonglong2*>(wp + j) = make_ulonglong2(u0, u1);
       }
       if (lane == 0) red[warp] = rsq;
       if (!__syncthreads_and(ok)) {  // a wait of this block has run out
@@ -367,66 +391,66 @@ __global__ void __launch_bounds__(kThreads, 1) aab_reg_kernel(const AabParams P,
 #pragma unroll
       for (int q = 0; q < NG; ++q) {
         const int gq = tid + kThreads * q;
-        if (gq < groups) {
-          float4 a[kWarps];
+        if (DP / 4 >= kThreads || gq < DP / 4) {
+          ulonglong2 a[kWarps];
 #pragma unroll
-          for (int v = 0; v < kWarps; ++v) a[v] = *reinterpret_cast<const float4*>(wpart + (size_t)v * dp + 4 * gq);
-          float4 u;
-          u.x = ((a[0].x + a[1].x) + (a[2].x + a[3].x)) + ((a[4].x + a[5].x) + (a[6].x + a[7].x));
-          u.y = ((a[0].y + a[1].y) + (a[2].y + a[3].y)) + ((a[4].y + a[5].y) + (a[6].y + a[7].y));
-          u.z = ((a[0].z + a[1].z) + (a[2].z + a[3].z)) + ((a[4].z + a[5].z) + (a[6].z + a[7].z));
-          u.w = ((a[0].w + a[1].w) + (a[2].w + a[3].w)) + ((a[4].w + a[5].w) + (a[6].w + a[7].w));
-          st_async_f4(u_dst[q], u, u_bar[q]);
+          for (int v = 0; v < kWarps; ++v) a[v] = *reinterpret_cast<const ulonglong2*>(wpart + v * DP + 4 * gq);
+          const P2 lo = p2_add(p2_add(p2_add(a[0].x, a[1].x), p2_add(a[2].x, a[3].x)),
+                               p2_add(p2_add(a[4].x, a[5].x), p2_add(a[6].x, a[7].x)));
+          const P2 hi = p2_add(p2_add(p2_add(a[0].y, a[1].y), p2_add(a[2].y, a[3].y)),
+                               p2_add(p2_add(a[4].y, a[5].y), p2_add(a[6].y, a[7].y)));
+          const float2 l = p2_unpack(lo), h = p2_unpack(hi);
+          st_async_f4(u_dst[q] + 4u * DP * par, make_float4(l.x, l.y, h.x, h.y), u_bar[q]);
         }
       }
-      if (warp == kWarps - 1 && lane < cl) {
-        const float r2 = ((red[0] + red[1]) + (red[2] + red[3])) + ((red[4] + red[5]) + (red[6] + red[7]));
-        st_async_f1(mapa_u32(smem_u32(rbuf + 16 * par + rank), (uint32_t)lane), r2, mapa_u32(a_barA, (uint32_t)lane));
-      }
+      if (warp == kWarps - 1 && lane < CL)
+        st_async_f1(r_dst + 64u * par, sum_n<kWarps>(red), r_bar);
       // ---- exchange A: u on the own slice, ρ²
       if (!mbar_wait_cluster(barA, par)) ok = false;
       if (tid == 0) mbar_arrive_expect_tx(barA, bytesA);
-      rho = sqrtf(sum16(rbuf + 16 * par, cl));
-      const float inv_rho = 1.0f / rho;
-      float4 vo[NG];
-      if (slice_warp) {  // θ v := SAᵀp − ρ v on the slice, SAᵀp = u/ρ
-        float zsq = 0.f;
+      P2 us[NQ][2];
+      if (slice_warp) {  // u on the slice: ranks in order, then the lanes of a group
 #pragma unroll
-        for (int q = 0; q < NG; ++q) {
-          const int gs = gsl + kThreads * q;
-          vo[q] = make_float4(zo[q].x * inv_theta, zo[q].y * inv_theta, zo[q].z * inv_theta, zo[q].w * inv_theta);
-          float4 u = make_float4(0.f, 0.f, 0.f, 0.f);
-          if (gs < ngr) {
-#pragma unroll 8
-            for (int b = hr0; b < hr1; ++b) {
-              const float4 a = *reinterpret_cast<const float4*>(ubuf + b * P.cols_per + 4 * gs);
-              u.x += a.x;
-              u.y += a.y;
-              u.z += a.z;
-              u.w += a.w;
-            }
+        for (int q = 0; q < NQ; ++q) {
+          ulonglong2 a[S::RPL];
+#pragma unroll
+          for (int e = 0; e < S::RPL; ++e)
+            a[e] = *reinterpret_cast<const ulonglong2*>(u_src + DP * par + e * S::COLS + 4 * kThreads * q);
+          us[q][0] = a[0].x;
+          us[q][1] = a[0].y;
+#pragma unroll
+          for (int e = 1; e < S::RPL; ++e) {
+            us[q][0] = p2_add(us[q][0], a[e].x);
+            us[q][1] = p2_add(us[q][1], a[e].y);
           }
-          for (int o = ng; o < 32; o <<= 1) {  // the H lanes of a group (none for ng ≥ 32)
-            u.x += __shfl_xor_sync(0xffffffffu, u.x, o);
-            u.y += __shfl_xor_sync(0xffffffffu, u.y, o);
-            u.z += __shfl_xor_sync(0xffffffffu, u.z, o);
-            u.w += __shfl_xor_sync(0xffffffffu, u.w, o);
-          }
-          zo[q].x = u.x * inv_rho - rho * vo[q].x;
-          zo[q].y = u.y * inv_rho - rho * vo[q].y;
-          zo[q].z = u.z * inv_rho - rho * vo[q].z;
-          zo[q].w = u.w * inv_rho - rho * vo[q].w;
-          if (gs < ngr) {
-            for (int b = hr0; b < hr1; ++b)
-              st_async_f4(mapa_u32(a_z + 16u * (uint32_t)(G0 + gs), (uint32_t)b), zo[q], mapa_u32(a_barB, (uint32_t)b));
-            if (hsh == 0)
-              zsq = fmaf(zo[q].x, zo[q].x, fmaf(zo[q].y, zo[q].y, fmaf(zo[q].z, zo[q].z, fmaf(zo[q].w, zo[q].w, zsq))));
+          if (!sums) us[q][0] = us[q][1] = 0ull;
+#pragma unroll
+          for (int o = S::NGS; o < 32; o <<= 1) {
+            us[q][0] = p2_add(us[q][0], __shfl_xor_sync(0xffffffffu, us[q][0], o));
+            us[q][1] = p2_add(us[q][1], __shfl_xor_sync(0xffffffffu, us[q][1], o));
           }
         }
-        zsq = warp_sum(zsq);
-        if (lane < cl)
-          st_async_f1(mapa_u32(a_tbuf + 4u * (rank * (uint32_t)nw + (uint32_t)warp), (uint32_t)lane), zsq,
-                      mapa_u32(a_barB, (uint32_t)lane));
+      }
+      float inv_rho;
+      norm_of(sum_n<CL>(rbuf + 16 * par), rho, inv_rho);
+      float4 vo[NQ];
+      if (slice_warp) {  // θ v := SAᵀp − ρ v on the slice, SAᵀp = u/ρ
+#pragma unroll
+        for (int q = 0; q < NQ; ++q) {
+          const float2 ul = p2_unpack(us[q][0]), uh = p2_unpack(us[q][1]);
+          vo[q] = make_float4(zo[q].x * inv_theta, zo[q].y * inv_theta, zo[q].z * inv_theta, zo[q].w * inv_theta);
+          zo[q].x = ul.x * inv_rho - rho * vo[q].x;
+          zo[q].y = ul.y * inv_rho - rho * vo[q].y;
+          zo[q].z = uh.x * inv_rho - rho * vo[q].z;
+          zo[q].w = uh.y * inv_rho - rho * vo[q].w;
+          if (sends) {
+#pragma unroll
+            for (int e = 0; e < S::SPL; ++e) {
+              const uint32_t to = (uint32_t)(sh * S::SPL + e);
+              st_async_f4(mapa_u32(z_src + 16u * kThreads * q, to), zo[q], mapa_u32(a_barB, to));
+            }
+          }
+        }
       }
       // ---- the recursion's scalars and the slice of d and x, while θv travels
       if (first) {
@@ -437,7 +461,7 @@ __global__ void __launch_bounds__(kThreads, 1) aab_reg_kernel(const AabParams P,
         const float inv = 1.0f / rhobar;
         if (slice_warp) {
 #pragma unroll
-          for (int q = 0; q < NG; ++q) {
+          for (int q = 0; q < NQ; ++q) {
             dv[q] = make_float4(vo[q].x * inv, vo[q].y * inv, vo[q].z * inv, vo[q].w * inv);
             xs[q] = make_float4(phi * dv[q].x, phi * dv[q].y, phi * dv[q].z, phi * dv[q].w);
           }
@@ -455,7 +479,7 @@ __global__ void __launch_bounds__(kThreads, 1) aab_reg_kernel(const AabParams P,
         phi = -phi * thetabar * inv_rhobar;
         if (slice_warp) {
 #pragma unroll
-          for (int q = 0; q < NG; ++q) {
+          for (int q = 0; q < NQ; ++q) {
             dv[q].x = (vo[q].x - thetabar * dv[q].x) * inv_rhobar;
             dv[q].y = (vo[q].y - thetabar * dv[q].y) * inv_rhobar;
             dv[q].z = (vo[q].z - thetabar * dv[q].z) * inv_rhobar;
@@ -471,16 +495,13 @@ __global__ void __launch_bounds__(kThreads, 1) aab_reg_kernel(const AabParams P,
       }
 #pragma unroll
       for (int r = 0; r < R; ++r) p[r] = w[r] * inv_rho;
-      // ---- exchange B: θv and θ² (also awaited before leaving: nothing may
+      // ---- exchange B: θv (also awaited before leaving: nothing may
       // still be on its way to a block that exits)
       if (!mbar_wait_cluster(barB, par)) ok = false;
       if (tid == 0) mbar_arrive_expect_tx(barB, bytesB);
       ok = __all_sync(0xffffffffu, ok);
       if (!ok) continue;  // to the block's next barrier, which sends every warp out
       if (!(t >= P.eps && k < P.max_passes && rho > 0.f)) break;  // the same in every block
-      theta = sqrtf(sum16(tbuf, cl * nw));
-      if (!(theta > 0.f)) break;  // invariant subspace: same decision everywhere
-      inv_theta = 1.0f / theta;
     }
     // Warps that left by the tests above meet, at this barrier, any warp of
     // the block whose wait ran out (its barrier is the one in the sweep).
@@ -498,14 +519,13 @@ __global__ void __launch_bounds__(kThreads, 1) aab_reg_kernel(const AabParams P,
   }
 
   // Outputs: each block writes its column slice.
-  if (slice_warp && hsh == 0) {
+  if (rep == 0 && hsh == 0) {
 #pragma unroll
-    for (int q = 0; q < NG; ++q) {
-      if (gsl + kThreads * q >= ngr) continue;
+    for (int q = 0; q < NQ; ++q) {
       const float xv[4] = {xs[q].x, xs[q].y, xs[q].z, xs[q].w};
 #pragma unroll
       for (int e = 0; e < 4; ++e) {
-        const int j = 4 * (G0 + gsl + kThreads * q) + e;
+        const int j = (int)rank * S::COLS + 4 * (gsl + kThreads * q) + e;
         if (j >= d) continue;
         const float dj = xv[e];
         if (delta_ != nullptr) delta_[j] = dj;
@@ -541,51 +561,44 @@ __global__ void __launch_bounds__(kThreads, 1) aab_reg_kernel(const AabParams P,
   cluster_wait();
 }
 
-using RegKernelFn = void (*)(const AabParams, int, int);
+// Rows per warp of the kernels: all steps for one block; only the upper half
+// for more (fewer rows would have fitted half the blocks).
+constexpr int reg_step(int ch) { return ch <= 2 ? 4 : (ch <= 4 ? 2 : 1); }
+constexpr int reg_max(int ch) { return ch == 16 ? 2 : 5 * reg_step(ch); }
 
-template <int CH>
-RegKernelFn reg_kernel_for_rows(int r) {
-  constexpr int step = CH <= 2 ? 4 : (CH <= 4 ? 2 : 1);  // kernels for R = step, 2·step, …
-  if constexpr (CH == 16) return r <= 1 ? aab_reg_kernel<16, 1> : aab_reg_kernel<16, 2>;
-  else {
-    if (r <= step) return aab_reg_kernel<CH, step>;
-    if (r <= 2 * step) return aab_reg_kernel<CH, 2 * step>;
-    if (r <= 3 * step) return aab_reg_kernel<CH, 3 * step>;
-    if (r <= 4 * step) return aab_reg_kernel<CH, 4 * step>;
-    return aab_reg_kernel<CH, 5 * step>;
+template <int CL, int CH>
+RegKernel reg_kernel_rows(int r) {
+  constexpr int st = reg_step(CH);
+  const size_t smem = RegShape<CL, CH>::bytes;
+  if constexpr (CH == 16) {
+    if constexpr (CL == 1) {
+      if (r <= 1) return {(const void*)aab_reg_kernel<CL, CH, 1>, smem};
+    }
+    return {(const void*)aab_reg_kernel<CL, CH, 2>, smem};
+  } else {
+    if constexpr (CL == 1) {
+      if (r <= st) return {(const void*)aab_reg_kernel<CL, CH, st>, smem};
+      if (r <= 2 * st) return {(const void*)aab_reg_kernel<CL, CH, 2 * st>, smem};
+    }
+    if (r <= 3 * st) return {(const void*)aab_reg_kernel<CL, CH, 3 * st>, smem};
+    if (r <= 4 * st) return {(const void*)aab_reg_kernel<CL, CH, 4 * st>, smem};
+    return {(const void*)aab_reg_kernel<CL, CH, 5 * st>, smem};
   }
 }
 
-RegKernelFn reg_kernel(int ch, int r) {
-  if (ch <= 2) return reg_kernel_for_rows<2>(r);
-  if (ch <= 4) return reg_kernel_for_rows<4>(r);
-  if (ch <= 8) return reg_kernel_for_rows<8>(r);
-  return reg_kernel_for_rows<16>(r);
+template <int CL>
+RegKernel reg_kernel_cl(int m, int dp) {
+  const int ch = (dp + 127) / 128, chp = ch <= 2 ? 2 : (ch <= 4 ? 4 : (ch <= 8 ? 8 : 16));
+  const int r = ((m + CL - 1) / CL + kWarps - 1) / kWarps;
+  if (r > reg_max(chp)) return {nullptr, 0};
+  switch (chp) {
+    case 2: return reg_kernel_rows<CL, 2>(r);
+    case 4: return reg_kernel_rows<CL, 4>(r);
+    case 8: return reg_kernel_rows<CL, 8>(r);
+    default: return reg_kernel_rows<CL, 16>(r);
+  }
 }
 
 }  // namespace
 }  // namespace aabk
-
-using namespace aabk;
-
-int aab_reg_device_error(int* code) {
-  int v = 0, zero = 0;
-  MIHS_CUDA_TRY(cudaMemcpyFromSymbol(&v, g_aab_reg_error, sizeof(int)));
-  if (v != 0) MIHS_CUDA_TRY(cudaMemcpyToSymbol(g_aab_reg_error, &zero, sizeof(int)));
-  *code = v;
-  return MIHS_OK;
-}
-
-int aabk::aab_reg_rows(int m, int cl, int dp) {
-  const int ch = (dp + 127) / 128;
-  const int chp = ch <= 2 ? 2 : (ch <= 4 ? 4 : (ch <= 8 ? 8 : 16));
-  const int rpc = (m + cl - 1) / cl;
-  const int r = (rpc + kWarps - 1) / kWarps;
-  return r * chp * 4 <= (chp == 16 ? 128 : 160) ? r : 0;
-}
-
-const void* aabk::aab_reg_fn(int dp, int r) { return (const void*)reg_kernel((dp + 127) / 128, r); }
-
-size_t aabk::aab_reg_smem(int dp, int cl, int cols_per) { return sizeof(float) * (size_t)reg_smem(dp, cl, cols_per).total; }
-
 }  // namespace mihs

@@ -258,6 +258,7 @@ struct mihs_sketch_s {
   // (P_path × 16 × dp), G and X⁻ (16 × dp each), 16 control blocks and the
   // path's stop counter / flag.
   void* aab_grid_ws = nullptr;   // global scratch of the single-λ grid AAb kernel (first solve that needs it)
+  int aab_grid_ws_type = 0, aab_grid_ws_blocks = 0;  // the launches it was prepared for
   int aab_form = MIHS_AAB_AUTO;  // form of AAb_Solver in single-λ solves (mihs_sketch_set_aab)
   int aab_grid_blocks = 0;
   float* path_partials = nullptr;
@@ -313,6 +314,7 @@ int use_grid_ws(mihs_sketch_s* sk, AabLaunch& a, cudaStream_t s) {
   a.aab_form = sk->aab_form;
   a.grid_blocks = sk->aab_grid_blocks;
   if (!aab_grid_wanted(a.m, a.d, a.sa_type, a.aab_form)) return MIHS_OK;
+  bool fresh = false;
   if (sk->aab_grid_ws == nullptr) {
     const size_t bytes = aab_grid_ws_bytes(a.d);
     cudaError_t e = cudaMalloc(&sk->aab_grid_ws, bytes);
@@ -321,8 +323,16 @@ int use_grid_ws(mihs_sketch_s* sk, AabLaunch& a, cudaStream_t s) {
       set_error("AAb grid scratch: cudaMalloc(%zu): %s", bytes, cudaGetErrorString(e));
       return e == cudaErrorMemoryAllocation ? MIHS_ERR_OOM : MIHS_ERR_CUDA;
     }
+    fresh = true;
   }
-  MIHS_CUDA_TRY(cudaMemsetAsync(sk->aab_grid_ws, 0, kAabGridBarBytes, s));
+  if (fresh || sk->aab_grid_ws_type != a.sa_type || sk->aab_grid_ws_blocks != a.grid_blocks) {
+    const int rc = aab_grid_ws_init(sk->aab_grid_ws, a.d, s);
+    if (rc) return rc;
+    sk->aab_grid_ws_type = a.sa_type;
+    sk->aab_grid_ws_blocks = a.grid_blocks;
+  } else {
+    MIHS_CUDA_TRY(cudaMemsetAsync(sk->aab_grid_ws, 0, kAabGridBarBytes, s));
+  }
   a.grid_ws = sk->aab_grid_ws;
   return MIHS_OK;
 }
@@ -332,7 +342,8 @@ int use_grid_scratch(AabLaunch& a, StreamScratch& ws, cudaStream_t s) {
   if (!aab_grid_wanted(a.m, a.d, a.sa_type)) return MIHS_OK;
   int rc = ws.alloc(aab_grid_ws_bytes(a.d), s);
   if (rc) return rc;
-  MIHS_CUDA_TRY(cudaMemsetAsync(ws.p, 0, kAabGridBarBytes, s));
+  rc = aab_grid_ws_init(ws.p, a.d, s);
+  if (rc) return rc;
   a.grid_ws = ws.p;
   return MIHS_OK;
 }
@@ -525,10 +536,12 @@ int mihs_device_status(int* code) {
   int gr = 0;
   rc = aab_grid_device_error(&gr);
   if (rc) return rc;
-  int re = 0;
+  int re = 0, gg = 0;
   rc = aab_reg_device_error(&re);
   if (rc) return rc;
-  *code = a ? a : (g ? g : (dd ? dd : (pa ? pa : (ab ? ab : (gr ? gr : re)))));
+  rc = aab_gridreg_device_error(&gg);
+  if (rc) return rc;
+  *code = a ? a : (g ? g : (dd ? dd : (pa ? pa : (ab ? ab : (gr ? gr : (re ? re : gg))))));
   return MIHS_OK;
 }
 

@@ -130,13 +130,23 @@ struct AabLaunch {
 // memory and a.grid_ws is given — one grid over the SMs (aab_grid.cu).
 int launch_aab(const AabLaunch& a, cudaStream_t s);
 // Single-λ AAb_Solver as one grid that keeps SA in the shared memory of up to
-// every SM.  `ws` holds aab_grid_ws_bytes(d) bytes whose first
-// kAabGridBarBytes hold the grid barrier word, which must be zero before a
-// solve (it returns to zero after every completed launch).  Returns
+// every SM.  `ws` holds aab_grid_ws_bytes(d) bytes prepared by
+// aab_grid_ws_init, whose first kAabGridBarBytes hold the grid barrier word,
+// which must be zero before a solve (it returns to zero after every completed
+// launch).  Returns
 // MIHS_ERR_UNSUPPORTED (nothing launched) when SA does not fit.
 constexpr size_t kAabGridBarBytes = 256;
 size_t aab_grid_ws_bytes(int d);
 int launch_aab_grid(const AabLaunch& a, void* ws, cudaStream_t s);
+// Makes freshly allocated scratch usable (and scratch whose next launches take
+// another block count or storage type than the last): clears the barrier word
+// and the tagged words of the register form (aab_grid_reg.cu).
+int aab_grid_ws_init(void* ws, int d, cudaStream_t s);
+// The register form of the grid, on its part of the scratch; UNSUPPORTED
+// (nothing launched) when `blocks` blocks do not hold SA in registers.
+int launch_aab_gridreg(const AabLaunch& a, int blocks, void* ws, cudaStream_t s);
+size_t aab_gridreg_ws_bytes(int d);
+int aab_gridreg_device_error(int* code);
 int aab_grid_device_error(int* code);
 int aab_reg_device_error(int* code);
 // True when launch_aab would take the grid form given scratch: `form` is
