@@ -36,11 +36,22 @@ template <int CH, int RW>
 __global__ void __launch_bounds__(kThreads, 1)
 apass_partial_kernel(const float* __restrict__ A, int n, int d, long long lda,
                      const float* __restrict__ b, const float* __restrict__ x,
+                     const double* __restrict__ x64, const double* __restrict__ xref,
                      float* __restrict__ partials, int dpad, int rows_per_cta, int stages,
-                     SolveCtl* __restrict__ ctl, int gate) {
+                     SolveCtl* __restrict__ ctl) {
   constexpr int NC = kConsumerWarps, R = NC * RW;
   constexpr bool XS = CH > 8;  // wide rows: keep x in smem instead of registers
-  if (ctl != nullptr && (ctl->done || (gate >= 0 && ctl_gate(ctl) != gate))) return;  // uniform
+  bool delta = false;  // a correction step of a refinement solve: x := x64 − xref, b := 0
+  if (ctl != nullptr) {  // uniform
+    if (ctl->done) return;
+    if (x64 != nullptr) {
+      const int gate = ctl_gate(ctl);
+      if (gate == 1) return;  // this step's gradient is the compensated one
+      delta = gate == 2;
+    }
+  }
+  if (delta) b = nullptr;
+  auto xval = [&](int j) { return delta ? (float)(x64[j] - xref[j]) : (x != nullptr ? x[j] : 0.f); };
   extern __shared__ __align__(128) unsigned char smem_raw[];
   float* ring = reinterpret_cast<float*>(smem_raw);
   uint64_t* full = reinterpret_cast<uint64_t*>(ring + (size_t)stages * R * dpad);
@@ -60,7 +71,7 @@ apass_partial_kernel(const float* __restrict__ A, int n, int d, long long lda,
     fence_mbar_init();
   }
   if (XS)
-    for (int j = threadIdx.x; j < CH * 128; j += kThreads) xsm[j] = (x != nullptr && j < d) ? x[j] : 0.f;
+    for (int j = threadIdx.x; j < CH * 128; j += kThreads) xsm[j] = j < d ? xval(j) : 0.f;
   __syncthreads();
 
   if (warp == NC) {  // ---------------------------------------------- producer
@@ -98,11 +109,11 @@ apass_partial_kernel(const float* __restrict__ A, int n, int d, long long lda,
     if (XS) continue;
     const int col = 4 * lane + 128 * c;
     float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
-    if (x != nullptr && col < d) {
-      v.x = x[col];
-      if (col + 1 < d) v.y = x[col + 1];
-      if (col + 2 < d) v.z = x[col + 2];
-      if (col + 3 < d) v.w = x[col + 3];
+    if (col < d) {
+      v.x = xval(col);
+      if (col + 1 < d) v.y = xval(col + 1);
+      if (col + 2 < d) v.z = xval(col + 2);
+      if (col + 3 < d) v.w = xval(col + 3);
     }
     xr[XS ? 0 : c] = v;
   }
@@ -186,29 +197,32 @@ apass_partial_kernel(const float* __restrict__ A, int n, int d, long long lda,
   }
 }
 
-// g[j] = Σ_p partials[p][j] − λ x[j]; 32 columns × 8 partial groups per block.
+// g[j] = Σ_p partials[p][j] − λ x[j] in a fixed order.  8 columns × 32 partial
+// groups per block: at most five loads per thread, all in flight at once (32
+// columns × 8 groups walked 19 partials each on a quarter of the blocks), then
+// one warp per column adds the groups.
 __global__ void __launch_bounds__(256)
 apass_finalize_kernel(const float* __restrict__ partials, int P, int d, int dpad,
                       const float* __restrict__ x, float lambda, const float* __restrict__ rhs,
-                      float* __restrict__ g, const SolveCtl* __restrict__ ctl, int gate,
-                      const double* __restrict__ base64) {
-  if (ctl != nullptr && (ctl->done || (gate >= 0 && ctl_gate(ctl) != gate))) return;
-  __shared__ float red[8][33];
-  const int lane = threadIdx.x & 31, grp = threadIdx.x >> 5;
-  const int j = blockIdx.x * 32 + lane;
+                      float* __restrict__ g, const SolveCtl* __restrict__ ctl) {
+  if (ctl != nullptr && ctl->done) return;
+  __shared__ float red[32][9];
+  const int c = threadIdx.x & 7, grp = threadIdx.x >> 3;
+  const int col = blockIdx.x * 8 + c;
   float s = 0.f;
-  if (j < d) {
-    for (int p = grp; p < P; p += 8) s += partials[(size_t)p * dpad + j];
+  if (col < d) {
+#pragma unroll 8
+    for (int p = grp; p < P; p += 32) s += partials[(size_t)p * dpad + col];
   }
-  red[grp][lane] = s;
+  red[grp][c] = s;
   __syncthreads();
-  if (grp == 0 && j < d) {
-    float t = 0.f;
-#pragma unroll
-    for (int k = 0; k < 8; ++k) t += red[k][lane];
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const int j = blockIdx.x * 8 + warp;
+  float t = warp_sum(red[lane][warp]);
+  if (lane == 0 && j < d) {
     if (rhs != nullptr) t += rhs[j];
     t -= (x != nullptr ? lambda * x[j] : 0.f);
-    g[j] = base64 != nullptr ? (float)(base64[j] + (double)t) : t;
+    g[j] = t;
   }
 }
 
@@ -251,7 +265,8 @@ int apass_num_partials(int64_t n, int64_t d) {
 }
 
 int launch_apass_partial(const float* A, int64_t n, int64_t d, int64_t lda, const float* b,
-                         const float* x, float* partials, SolveCtl* ctl, cudaStream_t s, int gate) {
+                         const float* x, float* partials, SolveCtl* ctl, cudaStream_t s, const double* x64,
+                         const double* xref, int timer) {
   const ApassKernel k = pick(d);
   const int P = apass_num_partials(n, d);
   const int64_t dpad = apass_dpad(d);
@@ -266,9 +281,7 @@ int launch_apass_partial(const float* A, int64_t n, int64_t d, int64_t lda, cons
   int n32 = (int)n, d32 = (int)d, dp32 = (int)dpad;
   long long lda64 = lda;
   void* args[] = {(void*)&A, &n32, &d32, &lda64, (void*)&b, (void*)&x,
-                  (void*)&partials, &dp32, (void*)&rows_per_cta, &stages, (void*)&ctl, &gate};
-  // refinement corrections (gate 2) are timed apart from plain gradients
-  const int timer = gate == 2 ? kTimerApassCorr : kTimerApass;
+                  (void*)&x64, (void*)&xref, (void*)&partials, &dp32, (void*)&rows_per_cta, &stages, (void*)&ctl};
   timing_begin(timer, s);
   MIHS_CUDA_TRY(cudaLaunchKernel(k.fn, dim3(P), dim3(kThreads), args, smem, s));
   timing_end(timer, s);
@@ -285,11 +298,10 @@ int apass_device_error(int* code) {
 }
 
 int launch_apass_finalize(const float* partials, int P, int64_t d, const float* x,
-                          float lambda, float* g, const SolveCtl* ctl, cudaStream_t s, int gate,
-                          const float* rhs, const double* base64) {
+                          float lambda, float* g, const SolveCtl* ctl, cudaStream_t s, const float* rhs) {
   const int64_t dpad = apass_dpad(d);
-  apass_finalize_kernel<<<(unsigned)((d + 31) / 32), 256, 0, s>>>(partials, P, (int)d, (int)dpad,
-                                                                   x, lambda, rhs, g, ctl, gate, base64);
+  apass_finalize_kernel<<<(unsigned)((d + 7) / 8), 256, 0, s>>>(partials, P, (int)d, (int)dpad,
+                                                                   x, lambda, rhs, g, ctl);
   MIHS_CHECK_LAUNCH();
   count_launch();
   return MIHS_OK;

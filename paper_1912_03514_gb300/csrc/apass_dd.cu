@@ -304,33 +304,82 @@ apass_dd_kernel(const float* __restrict__ A, int n, int d, long long lda, const 
   }
 }
 
-// g[j] = Σ_p (hi + lo) − λ·x[j] in fp64 (fixed order); also an fp32 copy.
-__global__ void __launch_bounds__(256)
-apass_dd_finalize_kernel(const float2* __restrict__ partials, int P, int d, int dpad,
-                         const double* __restrict__ x, double lambda, double* __restrict__ g64,
-                         float* __restrict__ g32, const SolveCtl* __restrict__ ctl, int gate,
-                         const float* __restrict__ rhs, double* __restrict__ xref) {
-  if (ctl != nullptr && (ctl->done || (gate >= 0 && ctl_gate(ctl) != gate))) return;
-  __shared__ double red[8][33];
-  const int lane = threadIdx.x & 31, grp = threadIdx.x >> 5;
-  const int j = blockIdx.x * 32 + lane;
-  double s = 0.0;
-  if (j < d)
-    for (int p = grp; p < P; p += 8) {
-      const float2 v = partials[(size_t)p * dpad + j];
-      s += (double)v.x + (double)v.y;
+// g[j] = Σ_p (hi + lo) − λ·x[j] in fp64 (fixed order); also an fp32 copy.  8
+// columns × 32 partial groups per block: bound by the few fp64 units of an SM
+// (two additions and two conversions per partial), so the columns are spread
+// over as many SMs as there are (32 columns per block: 17 µs at d = 1024, now
+// 10).
+//
+// In a refinement solve this kernel finishes whichever gradient the step took
+// (ctl_gate): 0 the plain one (partials at x32), 1 the compensated one, kept
+// with x as (g_ref, x_ref), 2 the correction g = g_ref − H(x − x_ref) (partials
+// of H's first term at x − x_ref, b = 0).
+struct DdFinalizeArgs {
+  const float2* dd;        // P_dd × dpad pairs
+  int P_dd;
+  const float* partials;   // P × dpad (refinement solves)
+  int P;
+  int d, dpad;
+  const double* x;
+  const float* x32;
+  double lambda;
+  double* g64;
+  float* g32;
+  const float* rhs;
+  double* xref;
+  const SolveCtl* ctl;
+};
+
+__global__ void __launch_bounds__(256) apass_dd_finalize_kernel(const DdFinalizeArgs a) {
+  int gate = 1;
+  if (a.ctl != nullptr) {
+    if (a.ctl->done) return;
+    gate = ctl_gate(a.ctl);
+  }
+  __shared__ double red[32][9];
+  const int c = threadIdx.x & 7, grp = threadIdx.x >> 3;
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const int col = blockIdx.x * 8 + c, j = blockIdx.x * 8 + warp;
+  if (gate == 1) {
+    double s = 0.0;
+    if (col < a.d) {
+#pragma unroll 10
+      for (int p = grp; p < a.P_dd; p += 32) {
+        const float2 v = a.dd[(size_t)p * a.dpad + col];
+        s += (double)v.x + (double)v.y;
+      }
     }
-  red[grp][lane] = s;
-  __syncthreads();
-  if (grp == 0 && j < d) {
-    double t = 0.0;
+    red[grp][c] = s;
+    __syncthreads();
+    double t = red[lane][warp];
 #pragma unroll
-    for (int k = 0; k < 8; ++k) t += red[k][lane];
-    if (rhs != nullptr) t += (double)rhs[j];
-    if (x != nullptr) t -= lambda * x[j];
-    if (g64 != nullptr) g64[j] = t;
-    if (g32 != nullptr) g32[j] = (float)t;
-    if (xref != nullptr) xref[j] = x[j];  // the point this gradient was taken at
+    for (int o = 16; o > 0; o >>= 1) t += __shfl_xor_sync(0xffffffffu, t, o);
+    if (lane == 0 && j < a.d) {
+      if (a.rhs != nullptr) t += (double)a.rhs[j];
+      if (a.x != nullptr) t -= a.lambda * a.x[j];
+      if (a.g64 != nullptr) a.g64[j] = t;
+      if (a.g32 != nullptr) a.g32[j] = (float)t;
+      if (a.xref != nullptr) a.xref[j] = a.x[j];  // the point this gradient was taken at
+    }
+    return;
+  }
+  float s = 0.f;
+  if (col < a.d) {
+#pragma unroll 8
+    for (int p = grp; p < a.P; p += 32) s += a.partials[(size_t)p * a.dpad + col];
+  }
+  float(*redf)[9] = reinterpret_cast<float(*)[9]>(red);
+  redf[grp][c] = s;
+  __syncthreads();
+  float t = warp_sum(redf[lane][warp]);
+  if (lane == 0 && j < a.d) {
+    if (gate == 0) {
+      if (a.rhs != nullptr) t += a.rhs[j];
+      a.g32[j] = t - (float)a.lambda * a.x32[j];
+    } else {
+      t -= (float)a.lambda * (float)(a.x[j] - a.xref[j]);
+      a.g32[j] = (float)(a.g64[j] + (double)t);
+    }
   }
 }
 
@@ -398,10 +447,27 @@ int launch_apass_dd(const float* A, int64_t n, int64_t d, int64_t lda, const flo
 }
 
 int launch_apass_dd_finalize(const float2* partials, int P, int64_t d, const double* x, double lambda,
-                             double* g64, float* g32, const SolveCtl* ctl, cudaStream_t s, int gate,
-                             const float* rhs, double* xref) {
-  apass_dd_finalize_kernel<<<(unsigned)((d + 31) / 32), 256, 0, s>>>(partials, P, (int)d, (int)apass_dpad(d), x,
-                                                                     lambda, g64, g32, ctl, gate, rhs, xref);
+                             double* g64, cudaStream_t s) {
+  DdFinalizeArgs a = {};
+  a.dd = partials;
+  a.P_dd = P;
+  a.d = (int)d;
+  a.dpad = (int)apass_dpad(d);
+  a.x = x;
+  a.lambda = lambda;
+  a.g64 = g64;
+  apass_dd_finalize_kernel<<<(unsigned)((d + 7) / 8), 256, 0, s>>>(a);
+  MIHS_CHECK_LAUNCH();
+  count_launch();
+  return MIHS_OK;
+}
+
+int launch_refine_finalize(const float2* dd, int P_dd, const float* partials, int P, int64_t d, const double* x,
+                           const float* x32, double lambda, double* gref, double* xref, float* g,
+                           const float* rhs, const SolveCtl* ctl, cudaStream_t s) {
+  const DdFinalizeArgs a = {dd,     P_dd, partials, P, (int)d, (int)apass_dpad(d), x, x32,
+                            lambda, gref, g,        rhs, xref, ctl};
+  apass_dd_finalize_kernel<<<(unsigned)((d + 7) / 8), 256, 0, s>>>(a);
   MIHS_CHECK_LAUNCH();
   count_launch();
   return MIHS_OK;

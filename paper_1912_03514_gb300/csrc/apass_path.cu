@@ -271,20 +271,21 @@ __global__ void apass_path_finalize_kernel(const float* __restrict__ partials, i
   if (all_done != nullptr && *all_done) return;
   const int l = blockIdx.y;
   if (l >= sc.nl) return;
-  __shared__ float red[8][33];
-  const int lane = threadIdx.x & 31, grp = threadIdx.x >> 5;
-  const int j = blockIdx.x * 32 + lane;
+  __shared__ float red[32][9];  // 8 columns × 32 partial groups per block
+  const int c = threadIdx.x & 7, grp = threadIdx.x >> 3;
+  const int col = blockIdx.x * 8 + c;
   float s = 0.f;
-  if (j < d)
-    for (int p = grp; p < P; p += 8) s += partials[((size_t)p * kL + l) * dpad + j];
-  red[grp][lane] = s;
-  __syncthreads();
-  if (grp == 0 && j < d) {
-    float t = 0.f;
-#pragma unroll
-    for (int k = 0; k < 8; ++k) t += red[k][lane];
-    G[(long long)l * ldg + j] = t - (X != nullptr ? sc.lam[l] * X[(long long)l * ldx + j] : 0.f);
+  if (col < d) {
+#pragma unroll 8
+    for (int p = grp; p < P; p += 32) s += partials[((size_t)p * kL + l) * dpad + col];
   }
+  red[grp][c] = s;
+  __syncthreads();
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const int j = blockIdx.x * 8 + warp;
+  const float t = warp_sum(red[lane][warp]);
+  if (lane == 0 && j < d)
+    G[(long long)l * ldg + j] = t - (X != nullptr ? sc.lam[l] * X[(long long)l * ldx + j] : 0.f);
 }
 
 }  // namespace
@@ -329,7 +330,7 @@ int launch_apass_path(const float* A, int64_t n, int64_t d, int64_t lda, const f
 int launch_apass_path_finalize(const float* partials, int P, int64_t d, const float* X, int64_t ldx,
                                const PathScalars& sc, float* G, int64_t ldg, const int* all_done,
                                cudaStream_t s) {
-  apass_path_finalize_kernel<<<dim3((unsigned)((d + 31) / 32), (unsigned)sc.nl), 256, 0, s>>>(
+  apass_path_finalize_kernel<<<dim3((unsigned)((d + 7) / 8), (unsigned)sc.nl), 256, 0, s>>>(
       partials, P, (int)d, (int)apass_dpad(d), X, ldx, sc, G, ldg, all_done);
   MIHS_CHECK_LAUNCH();
   count_launch();

@@ -99,14 +99,6 @@ __global__ void ctl_init_kernel(SolveCtl* ctl, int max_outer, float tol, int pha
   *ctl = c;
 }
 
-// δ = x − x_ref in fp32 for the correction step of a refinement solve.
-__global__ void refine_delta_kernel(const double* __restrict__ x, const double* __restrict__ xref,
-                                    float* __restrict__ delta, int d, const SolveCtl* __restrict__ ctl) {
-  if (ctl->done || ctl_gate(ctl) != 2) return;
-  const int j = blockIdx.x * blockDim.x + threadIdx.x;
-  if (j < d) delta[j] = (float)(x[j] - xref[j]);
-}
-
 // λ-path control blocks: one per λ (plain solves), the stop counter cleared.
 __global__ void path_init_kernel(SolveCtl* ctl, int* cnt, int nl, int max_outer, float tol) {
   const int l = threadIdx.x;
@@ -211,7 +203,6 @@ struct mihs_sketch_s {
   float* bw32 = nullptr;  // 2·dp: fp32 roundings of x and v for refined backward solves
   double* gref64 = nullptr;  // dp: the compensated gradient at the last refresh
   double* xref64 = nullptr;  // dp: the point it was taken at
-  float* delta32 = nullptr;  // dp: x − x_ref for the fp32 correction pass
   int P_dd = 0;
   double last_sd = 0; // sd estimated by the last solve that was given sd ≤ 0
   SolveCtl* ctl;
@@ -378,41 +369,31 @@ void retire_graph(mihs_sketch_s* sk, cudaGraphExec_t& exec, cudaGraph_t& graph) 
 
 // One outer step of Algorithm 1 (gradient, partial-sum reduce, AAb_Solver +
 // heavy ball), plain fp32 or compensated (refinement).
-// In a refinement solve both gradient variants are launched, each gated on
-// ctl->phase (plain fp32 while it is 0, compensated once it is 1), unless
-// `phase` names the one the host knows to be current.
+// A refinement step has one of three gradients, by ctl_gate: the plain pass at
+// the fp32 shadow of x, a compensated refresh at x (kept with x as g_ref, x_ref)
+// or the correction g_ref − H(x − x_ref), whose product is a plain pass with
+// b = 0.  The plain pass kernel serves both its steps and one kernel finishes
+// all three, so a step launches four kernels of which one returns at once
+// (eight, five of them idle at 2.8 µs each, with a kernel per variant).
+// `phase`: the gate of the step when the host knows it.
 int launch_step(mihs_sketch_s* sk, const mihs_sketch_s::Key& key, const AabLaunch& a, bool refined,
                 cudaStream_t s, int phase = -1) {
   int rc = MIHS_OK;
   if (refined) {
-    // gate 0: plain fp32 pass at the fp32 shadow of x (phase 0)
-    if (phase < 0 || phase == 0) {
-      rc = launch_apass_partial(key.A, sk->n, sk->d, key.lda, key.b, sk->x32_shadow, sk->partials, sk->ctl, s, 0);
-      if (!rc) rc = launch_apass_finalize(sk->partials, sk->P, sk->d, sk->x32_shadow, (float)key.lam, sk->g,
-                                          sk->ctl, s, 0, key.rhs);
-    }
-    // gate 1: compensated refresh at x, kept with x as (g_ref, x_ref)
-    if (!rc && (phase < 0 || phase == 1)) {
-      const double* x64 = static_cast<const double*>(key.x);
+    const double* x64 = static_cast<const double*>(key.x);
+    if (phase != 1)
+      rc = launch_apass_partial(key.A, sk->n, sk->d, key.lda, key.b, sk->x32_shadow, sk->partials, sk->ctl, s, x64,
+                                sk->xref64, phase == 2 ? kTimerApassCorr : kTimerApass);
+    if (!rc && (phase < 0 || phase == 1))
       rc = launch_apass_dd(key.A, sk->n, sk->d, key.lda, key.b, x64, sk->dd_partials, sk->ctl, s, 1);
-      if (!rc) rc = launch_apass_dd_finalize(sk->dd_partials, sk->P_dd, sk->d, x64, key.lam, sk->gref64, sk->g,
-                                             sk->ctl, s, 1, key.rhs, sk->xref64);
-    }
-    // gate 2: g = g_ref − H(x − x_ref), H·δ by the fp32 pass with b = 0
-    if (!rc && (phase < 0 || phase == 2)) {
-      refine_delta_kernel<<<(unsigned)((sk->d + 255) / 256), 256, 0, s>>>(
-          static_cast<const double*>(key.x), sk->xref64, sk->delta32, (int)sk->d, sk->ctl);
-      MIHS_CHECK_LAUNCH();
-      count_launch();
-      rc = launch_apass_partial(key.A, sk->n, sk->d, key.lda, nullptr, sk->delta32, sk->partials, sk->ctl, s, 2);
-      if (!rc) rc = launch_apass_finalize(sk->partials, sk->P, sk->d, sk->delta32, (float)key.lam, sk->g,
-                                          sk->ctl, s, 2, nullptr, sk->gref64);
-    }
+    if (!rc)
+      rc = launch_refine_finalize(sk->dd_partials, sk->P_dd, sk->partials, sk->P, sk->d, x64, sk->x32_shadow, key.lam,
+                                  sk->gref64, sk->xref64, sk->g, key.rhs, sk->ctl, s);
   } else {
     rc = launch_apass_partial(key.A, sk->n, sk->d, key.lda, key.b, static_cast<const float*>(key.x),
                               sk->partials, sk->ctl, s);
     if (!rc) rc = launch_apass_finalize(sk->partials, sk->P, sk->d, static_cast<const float*>(key.x),
-                                        (float)key.lam, sk->g, sk->ctl, s, -1, key.rhs);
+                                        (float)key.lam, sk->g, sk->ctl, s, key.rhs);
   }
   if (!rc) rc = launch_aab(a, s);
   return rc;
@@ -998,7 +979,7 @@ static int solve_impl(mihs_sketch_t sk, const float* A, int64_t lda, const float
     sk->P_dd = apass_dd_num_partials(n, d);
     char* p = nullptr;
     const size_t bytes = sizeof(float2) * (size_t)sk->P_dd * sk->dp + 3 * sizeof(double) * (size_t)sk->dp +
-                         4 * sizeof(float) * (size_t)sk->dp;
+                         3 * sizeof(float) * (size_t)sk->dp;
     cudaError_t e = cudaMalloc(&p, bytes);
     if (e != cudaSuccess) {
       set_error("mihs_solve_refined: cudaMalloc(%zu): %s", bytes, cudaGetErrorString(e));
@@ -1010,7 +991,6 @@ static int solve_impl(mihs_sketch_t sk, const float* A, int64_t lda, const float
     sk->xref64 = sk->gref64 + sk->dp;
     sk->x32_shadow = reinterpret_cast<float*>(sk->xref64 + sk->dp);
     sk->bw32 = sk->x32_shadow + sk->dp;
-    sk->delta32 = sk->bw32 + 2 * sk->dp;
   }
   // sd ≤ 0: estimate it from SA (Algorithm 4 with the paper's T = 2,
   // ε_tr = 0.5); an over-estimate only slows the rate (Remark after
@@ -1047,7 +1027,7 @@ static int solve_impl(mihs_sketch_t sk, const float* A, int64_t lda, const float
     // ‖g(0)‖ (= ‖Aᵀb‖ for the ridge problem) for the relative residual.
     rc = launch_apass_partial(A, n, d, lda, b, nullptr, sk->partials, nullptr, s);
     if (rc) return rc;
-    rc = launch_apass_finalize(sk->partials, sk->P, d, nullptr, 0.f, sk->g, nullptr, s, -1, rhs);
+    rc = launch_apass_finalize(sk->partials, sk->P, d, nullptr, 0.f, sk->g, nullptr, s, rhs);
     if (rc) return rc;
     ctl_set_gnorm0_kernel<<<1, 256, 0, s>>>(sk->ctl, sk->g, (int)d);
     MIHS_CHECK_LAUNCH();
@@ -1143,7 +1123,7 @@ static int solve_impl(mihs_sketch_t sk, const float* A, int64_t lda, const float
   info->inner_iters_total = c.inner_total;
   info->rel_resid = c.gnorm0 > 0.f ? (double)c.gnorm / (double)c.gnorm0 : 0.0;
   info->status = c.done ? c.status : MIHS_NOT_CONVERGED;
-  if (graph_ran) count_launch((refined ? 8ull : 3ull) * (uint64_t)(c.outer + 1));
+  if (graph_ran) count_launch((refined ? 4ull : 3ull) * (uint64_t)(c.outer + 1));
   return info->status;
 }
 
@@ -1630,7 +1610,7 @@ int mihs_gradient_refined(const float* A, int64_t n, int64_t d, int64_t lda, con
   float2* part = static_cast<float2*>(scratch.p);
   rc = launch_apass_dd(A, n, d, lda, b, x, part, nullptr, s);
   if (rc) return rc;
-  return launch_apass_dd_finalize(part, P, d, x, lambda, g, nullptr, nullptr, s);
+  return launch_apass_dd_finalize(part, P, d, x, lambda, g, s);
 }
 
 }  // extern "C"

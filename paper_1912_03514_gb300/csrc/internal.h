@@ -18,18 +18,18 @@ inline int64_t apass_dpad(int64_t d) { return round_up(d, 4); }
 // may be NULL (taken as 0).  Skips all work when ctl != NULL and ctl->done.
 // A bounded wait that runs out sets ctl->status = MIHS_ERR_TIMEOUT and
 // ctl->done (when ctl != NULL) and the library-wide device error word.
-// gate ≥ 0: run only while ctl->phase == gate (refinement solves).
+// x64 (refinement solves): the pass runs in steps with ctl_gate 0, at x, and 2,
+// at x64 − xref with b = 0; steps with gate 1 take launch_apass_dd.
 int launch_apass_partial(const float* A, int64_t n, int64_t d, int64_t lda,
                          const float* b, const float* x, float* partials,
-                         SolveCtl* ctl, cudaStream_t s, int gate = -1);
+                         SolveCtl* ctl, cudaStream_t s, const double* x64 = nullptr,
+                         const double* xref = nullptr, int timer = 0 /* kTimerApass */);
 // Reads and clears the library-wide device error word (synchronises).
 int apass_device_error(int* code);
-// g[j] = rhs[j] + Σ_p partials[p][j] − λ·x[j] in a fixed order (rhs may be
-// null); with base64, g[j] = fp32(base64[j] + that) (refinement corrections).
+// g[j] = rhs[j] + Σ_p partials[p][j] − λ·x[j] in a fixed order (rhs may be null).
 int launch_apass_finalize(const float* partials, int P, int64_t d,
                           const float* x, float lambda, float* g,
-                          const SolveCtl* ctl, cudaStream_t s, int gate = -1,
-                          const float* rhs = nullptr, const double* base64 = nullptr);
+                          const SolveCtl* ctl, cudaStream_t s, const float* rhs = nullptr);
 
 // ---- λ-path gradient (apass_path.cu) ---------------------------------------
 // Per-λ scalars of a path solve (passed by value to the kernels).
@@ -80,12 +80,15 @@ int launch_backward_grads(const float* A, int64_t n, int64_t d, int64_t lda, con
 int apass_dd_num_partials(int64_t n, int64_t d);
 int launch_apass_dd(const float* A, int64_t n, int64_t d, int64_t lda, const float* b, const double* x,
                     float2* partials, SolveCtl* ctl, cudaStream_t s, int gate = -1);
-// g64[j] = rhs[j] + Σ_p (hi + lo) − λ·x[j] in fp64 (rhs may be null); g32
-// (optional) its fp32 rounding; xref (optional) receives x.  b of
-// launch_apass_dd may be null (taken as 0).
+// g64[j] = Σ_p (hi + lo) − λ·x[j] in fp64.  b of launch_apass_dd may be null
+// (taken as 0).
 int launch_apass_dd_finalize(const float2* partials, int P, int64_t d, const double* x, double lambda,
-                             double* g64, float* g32, const SolveCtl* ctl, cudaStream_t s, int gate = -1,
-                             const float* rhs = nullptr, double* xref = nullptr);
+                             double* g64, cudaStream_t s);
+// The gradient g (fp32) of a refinement step, whichever pass the step's gate
+// ran (see the kernel); gref and xref are the last refresh's.
+int launch_refine_finalize(const float2* dd, int P_dd, const float* partials, int P, int64_t d, const double* x,
+                           const float* x32, double lambda, double* gref, double* xref, float* g,
+                           const float* rhs, const SolveCtl* ctl, cudaStream_t s);
 int apass_dd_device_error(int* code);
 
 // ---- AAb_Solver (aab.cu) --------------------------------------------------

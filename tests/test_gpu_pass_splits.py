@@ -1,0 +1,77 @@
+"""The passes over A at the edges of their kernels' splits, on integer data: every sum is exact in fp32 in any
+order, so a dropped, doubled or misplaced row or column shows up as a difference."""
+import numpy as np
+import pytest
+import torch
+
+from paper_1912_03514_gb300 import mihs
+from paper_1912_03514_gb300 import workloads as W
+
+pytestmark = pytest.mark.gpu
+DEV = "cuda"
+
+
+def _matrix(n, d, seed, lo=-2, hi=2):
+    """A (n × d) with NaN between its rows, on the GPU, and its values in fp64."""
+    A = torch.full((n, (d + 3) // 4 * 4), float("nan"))
+    A[:, :d] = W.randint_matrix((n, d), seed, lo, hi)
+    return A.to(DEV)[:, :d], A[:, :d].double().numpy()
+
+
+# rows: less than a stage, one stage and one row more, more stages than the ring, rows that no block gets; columns:
+# one group, each width of the kernel, the last that takes 16 rows a stage and the first that takes 8
+@pytest.mark.parametrize("n,d,nl", [(3, 1, 1), (16, 64, 16), (17, 65, 3), (33, 128, 16), (3000, 127, 9),
+                                    (5000, 256, 16), (12000, 300, 2), (9000, 512, 16), (2500, 676, 16),
+                                    (2500, 700, 16), (2600, 704, 5), (4001, 1021, 16), (20001, 1024, 16)])
+def test_path_gradient_is_exact(n, d, nl):
+    A, An = _matrix(n, d, n + d)
+    b = W.randint_matrix((n,), 3, -9, 9)
+    X = W.randint_matrix((nl, d), 4, -1, 1)
+    lams = [float(l % 3) for l in range(nl)]
+    G = mihs.gradient_path(A, b.to(DEV), X.to(DEV), lams).cpu().double().numpy()
+    Xn = X.double().numpy()
+    ref = (b.double().numpy()[:, None] - An @ Xn.T).T @ An - np.array(lams)[:, None] * Xn
+    assert np.abs(ref).max() < 2 ** 24
+    assert np.array_equal(G, ref)
+    assert mihs.device_status() == 0
+
+
+# n, d: one group of columns and less, each width of the kernel with and without 16-byte rows of dA, staged in two
+# halves past 1024 columns, the last row's last group
+@pytest.mark.parametrize("n,d", [(1, 1), (5, 3), (64, 4), (33, 127), (100, 129), (257, 255), (300, 512), (301, 510),
+                                 (77, 1001), (129, 1024), (65, 1025), (40, 2047), (41, 2048)])
+def test_backward_is_exact(n, d):
+    A, An = _matrix(n, d, 5 * n + d)
+    b, x, v = W.randint_matrix((n,), 6, -9, 9), W.randint_matrix((d,), 7, -2, 2), W.randint_matrix((d,), 8, -2, 2)
+    off = torch.zeros(d + 1, device=DEV)  # x not 16-byte aligned
+    off[1:] = x.to(DEV)
+    bn, xn, vn = (t.double().numpy() for t in (b, x, v))
+    r, q = bn - An @ xn, An @ vn
+    dA, db, dl = mihs.backward_grads(A, b.to(DEV), off[1:], v.to(DEV))
+    assert np.array_equal(dA.cpu().double().numpy(), np.outer(r, vn) - np.outer(q, xn))
+    assert np.array_equal(db.cpu().double().numpy(), q)
+    assert float(dl) == -float(xn @ vn)
+    _, db2, _ = mihs.backward_grads(A, b.to(DEV), off[1:], v.to(DEV), want_dA=False)
+    assert torch.equal(db, db2)
+
+
+# n, d: fewer rows than a split or a quad, a last split that is shorter, one and several column slices, ragged columns
+@pytest.mark.parametrize("n,d", [(1, 1), (3, 7), (5, 1030), (33, 4096), (37, 8193), (130, 50001), (513, 20000),
+                                 (2048, 2048), (2045, 9001)])
+def test_dual_gradient_is_exact(n, d):
+    A, An = _matrix(n, d, 9 * n + d, -1, 1)
+    b, nu = W.randint_matrix((n,), 10, -9, 9), W.randint_matrix((n,), 11, -1, 1)
+    g = mihs.gradient_dual(A, b.to(DEV), nu.to(DEV), 2.0).cpu().double().numpy()
+    u = An.T @ nu.double().numpy()
+    assert np.array_equal(g, b.double().numpy() - An @ u - 2.0 * nu.double().numpy())
+    assert np.array_equal(mihs.dual_recover(A, nu.to(DEV)).cpu().double().numpy(), u)
+
+
+@pytest.mark.parametrize("n,d", [(1, 1), (9, 8), (40, 9), (3000, 257), (5000, 2048)])
+def test_gradients_are_exact(n, d):
+    """The split-K reductions: fewer and more partials than groups, columns past the last block."""
+    A, An = _matrix(n, d, 13 * n + d)
+    b, x = W.randint_matrix((n,), 14, -9, 9), W.randint_matrix((d,), 15, -1, 1)
+    ref = An.T @ (b.double().numpy() - An @ x.double().numpy()) - 3.0 * x.double().numpy()
+    assert np.array_equal(mihs.gradient(A, b.to(DEV), x.to(DEV), 3.0).cpu().double().numpy(), ref)
+    assert np.array_equal(mihs.gradient_refined(A, b.to(DEV), x.double().to(DEV), 3.0).cpu().numpy(), ref)
