@@ -522,7 +522,10 @@ int mihs_device_status(int* code) {
   if (rc) return rc;
   rc = aab_gridreg_device_error(&gg);
   if (rc) return rc;
-  *code = a ? a : (g ? g : (dd ? dd : (pa ? pa : (ab ? ab : (gr ? gr : (re ? re : gg))))));
+  int du = 0;
+  rc = dual_device_error(&du);
+  if (rc) return rc;
+  *code = a ? a : (g ? g : (dd ? dd : (pa ? pa : (ab ? ab : (gr ? gr : (re ? re : (gg ? gg : du)))))));
   return MIHS_OK;
 }
 

@@ -49,52 +49,117 @@ __global__ void transpose_kernel(const float* __restrict__ A, int n, int d, long
 }
 
 // Partial u over a row split: part[z][j] = Σ_{i in split z} ν_i A[i][j].  A
-// thread owns 4 consecutive columns (one float4 per row, coalesced across the
-// warp) and walks its split's rows in order, eight rows of loads in flight.
-constexpr int kAtnuRows = 256;  // rows per split
+// block owns 1024 columns; a producer lane group streams their 4 KB of each
+// row into a shared-memory ring (bulk copies, completion counted in bytes) and
+// each of 256 consumer threads owns 4 columns and adds the rows in order.
+//
+// HBM-bound (4·n·d bytes).  Plain 16-byte loads reached the measured bandwidth
+// only where rows start on 128-byte lines: at 2000×200001 (rows 16 bytes off
+// from one to the next) a warp's 512 bytes lie on five lines instead of four
+// and the pass took 330 µs (5.0 TB/s) against 235 at 2000×200000; bulk copies
+// need no alignment beyond 16 bytes.  Up to kAtnuRows rows per split, fewer
+// where the columns alone do not make several waves of blocks.
+constexpr int kAtnuRows = 256;
+constexpr int kAtnuCols = 4 * kT;       // columns per block
+constexpr int kAtnuStageRows = 8;       // 32 KB per stage
+constexpr int kAtnuStages = 3;          // two blocks per SM
+constexpr size_t kAtnuSmem = sizeof(float) * (size_t)kAtnuStages * kAtnuStageRows * kAtnuCols;
 
-__global__ void __launch_bounds__(kT) atnu_partial_kernel(const float* __restrict__ A, int n, int d, long long lda,
-                                                          const float* __restrict__ nu, float* __restrict__ part,
-                                                          long long ldp, const SolveCtl* __restrict__ ctl) {
+__device__ int g_dual_error = 0;
+
+__global__ void __launch_bounds__(kT + 32, 2)
+atnu_partial_kernel(const float* __restrict__ A, int n, int d, long long lda, const float* __restrict__ nu,
+                    float* __restrict__ part, long long ldp, int rows, SolveCtl* __restrict__ ctl) {
   if (ctl != nullptr && ctl->done) return;
+  extern __shared__ __align__(128) float ring[];
   __shared__ float nus[kAtnuRows];
-  const int i0 = blockIdx.y * kAtnuRows, i1 = min(n, i0 + kAtnuRows);
-  for (int i = i0 + threadIdx.x; i < i1; i += kT) nus[i - i0] = nu[i];
+  __shared__ uint64_t full[kAtnuStages], empty[kAtnuStages];
+  __shared__ volatile int issued;  // stages sent for (for the abort path)
+  const int tid = threadIdx.x, lane = tid & 31;
+  const int i0 = blockIdx.y * rows, i1 = min(n, i0 + rows);
+  const int nst = (i1 - i0 + kAtnuStageRows - 1) / kAtnuStageRows;
+  const long long c0 = (long long)blockIdx.x * kAtnuCols;
+  // whole groups of four columns come through the ring; the last d mod 4 by plain loads
+  const int cols = (int)min((long long)kAtnuCols, (d & ~3ll) - c0);  // may be ≤ 0
+  if (tid == 0) {
+    for (int q = 0; q < kAtnuStages; ++q) {
+      mbar_init(&full[q], 1);
+      mbar_init(&empty[q], kT / 32);
+    }
+    issued = 0;
+    fence_mbar_init();
+  }
+  for (int i = i0 + tid; i < i1; i += kT + 32) nus[i - i0] = nu[i];
   __syncthreads();
-  const long long c = ((long long)blockIdx.x * kT + threadIdx.x) * 4;
-  if (c >= d) return;
-  float* out = part + (long long)blockIdx.y * ldp + c;
-  if (c + 4 <= d) {
+
+  if (tid >= kT) {  // producer warp: one lane per row of the stage
+    if (cols <= 0) return;
+    for (int it = 0; it < nst; ++it) {
+      const int q = it % kAtnuStages;
+      bool ok = true;
+      if (it >= kAtnuStages) {
+        if (lane == 0) ok = mbar_wait(&empty[q], ((uint32_t)(it / kAtnuStages) & 1u) ^ 1u, kWaitLimitNs);
+        ok = __shfl_sync(0xffffffffu, ok, 0);
+      }
+      if (!ok) {
+        if (lane == 0) atomicExch(&g_dual_error, MIHS_ERR_TIMEOUT);
+        break;
+      }
+      const int row0 = i0 + it * kAtnuStageRows, nrow = min(kAtnuStageRows, i1 - row0);
+      if (lane == 0) mbar_arrive_expect_tx(&full[q], (uint32_t)(nrow * cols) * 4u);
+      __syncwarp();
+      if (lane < nrow)
+        bulk_copy_g2s(ring + ((size_t)q * kAtnuStageRows + lane) * kAtnuCols, A + (row0 + lane) * lda + c0,
+                      (uint32_t)cols * 4u, &full[q]);
+      if (lane == 0) issued = it + 1;
+    }
+    return;
+  }
+
+  float* out = part + (long long)blockIdx.y * ldp + c0 + 4 * tid;
+  if (cols > 0) {
     float4 acc = make_float4(0.f, 0.f, 0.f, 0.f);
-    const float* col = A + c;
-    int i = i0;
-    for (; i + 8 <= i1; i += 8) {
-      float4 a[8];
+    int it = 0;
+    for (; it < nst; ++it) {
+      const int q = it % kAtnuStages;
+      if (!mbar_wait(&full[q], (uint32_t)(it / kAtnuStages) & 1u, kWaitLimitNs)) {
+        atomicExch(&g_dual_error, MIHS_ERR_TIMEOUT);
+        break;
+      }
+      const float* st = ring + (size_t)q * kAtnuStageRows * kAtnuCols + 4 * tid;
+      const int row0 = it * kAtnuStageRows, nrow = min(kAtnuStageRows, i1 - i0 - row0);
+      auto add = [&](int r) {
+        const float4 a = *reinterpret_cast<const float4*>(st + (size_t)r * kAtnuCols);
+        const float s = nus[row0 + r];
+        acc.x = fmaf(s, a.x, acc.x);
+        acc.y = fmaf(s, a.y, acc.y);
+        acc.z = fmaf(s, a.z, acc.z);
+        acc.w = fmaf(s, a.w, acc.w);
+      };
+      if (nrow == kAtnuStageRows) {
 #pragma unroll
-      for (int k = 0; k < 8; ++k) a[k] = __ldg(reinterpret_cast<const float4*>(col + (long long)(i + k) * lda));
-#pragma unroll
-      for (int k = 0; k < 8; ++k) {
-        const float s = nus[i + k - i0];
-        acc.x = fmaf(s, a[k].x, acc.x);
-        acc.y = fmaf(s, a[k].y, acc.y);
-        acc.z = fmaf(s, a[k].z, acc.z);
-        acc.w = fmaf(s, a[k].w, acc.w);
+        for (int r = 0; r < kAtnuStageRows; ++r) add(r);
+      } else {
+        for (int r = 0; r < nrow; ++r) add(r);
+      }
+      __syncwarp();
+      if (lane == 0) mbar_arrive(&empty[q]);
+    }
+    if (it < nst && tid == 0) {  // aborted: let the copies under way land before the block exits
+      for (int e = it; e < issued; ++e)
+        if (!mbar_wait(&full[e % kAtnuStages], (uint32_t)(e / kAtnuStages) & 1u, kWaitLimitNs)) break;
+      if (ctl != nullptr) {
+        ctl->status = MIHS_ERR_TIMEOUT;
+        ctl->done = 1;
       }
     }
-    for (; i < i1; ++i) {
-      const float4 a = __ldg(reinterpret_cast<const float4*>(col + (long long)i * lda));
-      const float s = nus[i - i0];
-      acc.x = fmaf(s, a.x, acc.x);
-      acc.y = fmaf(s, a.y, acc.y);
-      acc.z = fmaf(s, a.z, acc.z);
-      acc.w = fmaf(s, a.w, acc.w);
-    }
-    *reinterpret_cast<float4*>(out) = acc;
-  } else {
-    float t[3] = {0.f, 0.f, 0.f};
-    for (int i = i0; i < i1; ++i)
-      for (int k = 0; k < 3 && c + k < d; ++k) t[k] = fmaf(nus[i - i0], A[(long long)i * lda + c + k], t[k]);
-    for (int k = 0; k < 3 && c + k < d; ++k) out[k] = t[k];
+    if (4 * tid < cols) *reinterpret_cast<float4*>(out) = acc;
+  }
+  const long long c = (d & ~3ll) + tid;  // the last d mod 4 columns, by the block they fall in
+  if (c < d && c >= c0 && c < c0 + kAtnuCols) {
+    float t = 0.f;
+    for (int i = i0; i < i1; ++i) t = fmaf(nus[i - i0], A[(long long)i * lda + c], t);
+    part[(long long)blockIdx.y * ldp + c] = t;
   }
 }
 
@@ -109,25 +174,30 @@ __global__ void atnu_reduce_kernel(const float* __restrict__ part, int nsplit, l
   u[j] = t;
 }
 
-// g_i = b_i − A_i·u − λν_i for kRowsPerBlock rows per block (each load of u
-// serves them all), fixed-order block sums.
+// A_i·u over a column slice for kResidRows rows per block (each load of u
+// serves them all), fixed-order block sums: part[slice][i], or with one slice
+// g_i = b_i − A_i·u − λν_i at once.  Slices only where four rows per block do
+// not make three blocks per SM (128×200000: 32 blocks, both passes 183 µs; cut
+// into slices, with the other pass below its 30 µs of HBM time, 47 µs).
 constexpr int kResidRows = 4;
 
 __global__ void __launch_bounds__(kT) dual_resid_kernel(const float* __restrict__ A, int n, int d, long long lda,
                                                         const float* __restrict__ u, const float* __restrict__ b,
-                                                        const float* __restrict__ nu, float lam,
-                                                        float* __restrict__ g, const SolveCtl* __restrict__ ctl) {
+                                                        const float* __restrict__ nu, float lam, int cols,
+                                                        float* __restrict__ part, float* __restrict__ g,
+                                                        const SolveCtl* __restrict__ ctl) {
   if (ctl != nullptr && ctl->done) return;
   __shared__ float red[kResidRows][kT / 32];
-  const int i0 = blockIdx.x * kResidRows;
-  const int d4 = d >> 2;
+  const int i0 = blockIdx.y * kResidRows;
+  const int k0 = blockIdx.x * (cols >> 2), k1 = min(d >> 2, k0 + (cols >> 2));
   float s0[kResidRows], s1[kResidRows];
 #pragma unroll
   for (int r = 0; r < kResidRows; ++r) s0[r] = s1[r] = 0.f;
   const float* rows[kResidRows];
 #pragma unroll
   for (int r = 0; r < kResidRows; ++r) rows[r] = A + (long long)min(i0 + r, n - 1) * lda;
-  for (int k = threadIdx.x; k < d4; k += kT) {
+#pragma unroll 2
+  for (int k = k0 + threadIdx.x; k < k1; k += kT) {
     const float4 v = __ldcg(reinterpret_cast<const float4*>(u) + k);
 #pragma unroll
     for (int r = 0; r < kResidRows; ++r) {
@@ -136,10 +206,11 @@ __global__ void __launch_bounds__(kT) dual_resid_kernel(const float* __restrict_
       s1[r] = fmaf(a.y, v.y, fmaf(a.w, v.w, s1[r]));
     }
   }
-  for (int j = 4 * d4 + threadIdx.x; j < d; j += kT) {
+  if (blockIdx.x == gridDim.x - 1)  // the ragged last columns
+    for (int j = 4 * (d >> 2) + threadIdx.x; j < d; j += kT) {
 #pragma unroll
-    for (int r = 0; r < kResidRows; ++r) s0[r] = fmaf(rows[r][j], u[j], s0[r]);
-  }
+      for (int r = 0; r < kResidRows; ++r) s0[r] = fmaf(rows[r][j], u[j], s0[r]);
+    }
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
 #pragma unroll
   for (int r = 0; r < kResidRows; ++r) {
@@ -152,8 +223,26 @@ __global__ void __launch_bounds__(kT) dual_resid_kernel(const float* __restrict_
     float t = 0.f;
 #pragma unroll
     for (int w = 0; w < kT / 32; ++w) t += red[r][w];
-    if (i < n) g[i] = b[i] - t - (nu != nullptr ? lam * nu[i] : 0.f);
+    if (i < n) {
+      if (gridDim.x == 1)
+        g[i] = b[i] - t - (nu != nullptr ? lam * nu[i] : 0.f);
+      else
+        part[(size_t)blockIdx.x * n + i] = t;
+    }
   }
+}
+
+// g_i = b_i − Σ_slices part[slice][i] − λν_i in order of the slices.
+__global__ void dual_resid_finish_kernel(const float* __restrict__ part, int slices, int n, const float* __restrict__ b,
+                                         const float* __restrict__ nu, float lam, float* __restrict__ g,
+                                         const SolveCtl* __restrict__ ctl) {
+  if (ctl != nullptr && ctl->done) return;
+  const int i = blockIdx.x * blockDim.x + threadIdx.x;
+  if (i >= n) return;
+  float t = 0.f;
+#pragma unroll 8
+  for (int z = 0; z < slices; ++z) t += part[(size_t)z * n + i];
+  g[i] = b[i] - t - (nu != nullptr ? lam * nu[i] : 0.f);
 }
 
 __global__ void dual_ctl_init_kernel(SolveCtl* ctl, int max_outer, float tol) {
@@ -177,28 +266,65 @@ __global__ void dual_gnorm0_kernel(SolveCtl* ctl, const float* b, int n) {
   }
 }
 
-int atnu_num_splits(int64_t n) { return (int)((n + kAtnuRows - 1) / kAtnuRows); }
+// Cuts of the two passes over A (column slices of A·u for a matrix with too few
+// rows to fill the GPU).
+struct DualPlan {
+  int rows, splits;    // Aᵀν: rows per split
+  int cols, slices;    // A·u: column slices (cols a multiple of 4)
+};
+DualPlan dual_plan(int64_t n, int64_t d) {
+  DualPlan p;
+  const int64_t cblocks = (d + kAtnuCols - 1) / kAtnuCols;
+  int64_t splits = (8LL * num_sms() + cblocks - 1) / cblocks;  // four waves of two blocks per SM
+  if (splits > (n + 31) / 32) splits = (n + 31) / 32;          // of at least 32 rows each
+  p.rows = (int)round_up((n + splits - 1) / splits, kAtnuStageRows);
+  if (p.rows > kAtnuRows) p.rows = kAtnuRows;
+  p.splits = (int)((n + p.rows - 1) / p.rows);
+  const int64_t quads = (n + kResidRows - 1) / kResidRows;
+  int64_t slices = quads >= 3LL * num_sms() ? 1 : (4LL * num_sms() + quads - 1) / quads;
+  if (slices > d / 4096) slices = d / 4096;                 // at least 16 KB of a row each
+  if (slices < 1) slices = 1;
+  p.cols = (int)round_up((d + slices - 1) / slices, 4);
+  p.slices = (int)((d + p.cols - 1) / p.cols);
+  return p;
+}
 
-// u = Aᵀν through row-split partials `part` (atnu_num_splits(n) × round_up(d, 4) floats).
-int launch_atnu(const float* A, int64_t n, int64_t d, int64_t lda, const float* nu, float* u, float* part,
-                const SolveCtl* ctl, cudaStream_t s) {
-  const int ns = atnu_num_splits(n);
+// Scratch of both passes: Aᵀν's row-split partials (splits × round_up(d, 4)),
+// then A·u's column-slice partials (slices × n).
+size_t dual_scratch_floats(int64_t n, int64_t d) {
+  const DualPlan p = dual_plan(n, d);
+  return (size_t)p.splits * (size_t)round_up(d, 4) + (size_t)p.slices * (size_t)round_up(n, 4);
+}
+
+// u = Aᵀν through row-split partials in `scratch`.
+int launch_atnu(const float* A, int64_t n, int64_t d, int64_t lda, const float* nu, float* u, float* scratch,
+                SolveCtl* ctl, cudaStream_t s) {
+  const DualPlan p = dual_plan(n, d);
   const long long ldp = round_up(d, 4);
-  const unsigned cblocks = (unsigned)((d + 4 * kT - 1) / (4 * kT));
-  atnu_partial_kernel<<<dim3(cblocks, (unsigned)ns), kT, 0, s>>>(A, (int)n, (int)d, lda, nu, part, ldp, ctl);
+  const unsigned cblocks = (unsigned)((d + kAtnuCols - 1) / kAtnuCols);
+  MIHS_CUDA_TRY(cudaFuncSetAttribute(atnu_partial_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kAtnuSmem));
+  atnu_partial_kernel<<<dim3(cblocks, (unsigned)p.splits), kT + 32, kAtnuSmem, s>>>(A, (int)n, (int)d, lda, nu, scratch,
+                                                                                    ldp, p.rows, ctl);
   MIHS_CHECK_LAUNCH();
-  atnu_reduce_kernel<<<(unsigned)((d + 255) / 256), 256, 0, s>>>(part, ns, ldp, (int)d, u, ctl);
+  atnu_reduce_kernel<<<(unsigned)((d + 255) / 256), 256, 0, s>>>(scratch, p.splits, ldp, (int)d, u, ctl);
   MIHS_CHECK_LAUNCH();
   count_launch(2);
   return MIHS_OK;
 }
 
 int launch_dual_resid(const float* A, int64_t n, int64_t d, int64_t lda, const float* u, const float* b,
-                      const float* nu, float lam, float* g, const SolveCtl* ctl, cudaStream_t s) {
-  dual_resid_kernel<<<(unsigned)((n + kResidRows - 1) / kResidRows), kT, 0, s>>>(A, (int)n, (int)d, lda, u, b, nu,
-                                                                                 lam, g, ctl);
+                      const float* nu, float lam, float* g, float* scratch, const SolveCtl* ctl, cudaStream_t s) {
+  const DualPlan p = dual_plan(n, d);
+  float* part = scratch + (size_t)p.splits * (size_t)round_up(d, 4);
+  dual_resid_kernel<<<dim3((unsigned)p.slices, (unsigned)((n + kResidRows - 1) / kResidRows)), kT, 0, s>>>(
+      A, (int)n, (int)d, lda, u, b, nu, lam, p.cols, part, g, ctl);
   MIHS_CHECK_LAUNCH();
   count_launch();
+  if (p.slices > 1) {
+    dual_resid_finish_kernel<<<(unsigned)((n + 127) / 128), 128, 0, s>>>(part, p.slices, (int)n, b, nu, lam, g, ctl);
+    MIHS_CHECK_LAUNCH();
+    count_launch();
+  }
   return MIHS_OK;
 }
 
@@ -215,13 +341,21 @@ int check_dual(const float* A, int64_t n, int64_t d, int64_t lda, const char* wh
 
 }  // namespace
 
+int mihs::dual_device_error(int* code) {
+  int v = 0, zero = 0;
+  MIHS_CUDA_TRY(cudaMemcpyFromSymbol(&v, g_dual_error, sizeof(int)));
+  if (v != 0) MIHS_CUDA_TRY(cudaMemcpyToSymbol(g_dual_error, &zero, sizeof(int)));
+  *code = v;
+  return MIHS_OK;
+}
+
 struct mihs_dual_s {
   int64_t n, d, m, np;
   int family;
   uint64_t seed;
   float* SAt = nullptr;   // m × np
   float* u = nullptr;     // d
-  float* upart = nullptr; // atnu_num_splits(n) × round_up(d, 4): row-split partials of Aᵀν
+  float* upart = nullptr; // dual_scratch_floats(n, d): partials of the two passes over A
   float* g = nullptr;     // np
   float* nu_prev = nullptr;  // np
   void* grid_ws = nullptr;   // scratch of the grid form of AAb_Solver (first solve that needs it)
@@ -265,7 +399,7 @@ int dual_sketch_into(mihs_dual_t dk, const float* A, int64_t lda, uint64_t seed,
 // One step of Algorithm 2 (both gradient passes and the AAb + heavy ball).
 int dual_step(mihs_dual_t dk, const mihs_dual_s::Key& k, const AabLaunch& a, cudaStream_t s) {
   int rc = launch_atnu(k.A, dk->n, dk->d, k.lda, k.nu, dk->u, dk->upart, dk->ctl, s);
-  if (!rc) rc = launch_dual_resid(k.A, dk->n, dk->d, k.lda, dk->u, k.b, k.nu, (float)k.lam, dk->g, dk->ctl, s);
+  if (!rc) rc = launch_dual_resid(k.A, dk->n, dk->d, k.lda, dk->u, k.b, k.nu, (float)k.lam, dk->g, dk->upart, dk->ctl, s);
   if (!rc) rc = launch_aab(a, s);
   return rc;
 }
@@ -347,7 +481,7 @@ int mihs_dual_sketch(const float* A, int64_t n, int64_t d, int64_t lda, int fami
   dk->family = family;
   char* p = nullptr;
   const size_t fl = (size_t)m * dk->np + (size_t)round_up(d, 4) + 2 * (size_t)dk->np +
-                    (size_t)atnu_num_splits(n) * (size_t)round_up(d, 4);
+                    dual_scratch_floats(n, d);
   cudaError_t e = cudaMalloc(&p, fl * sizeof(float) + sizeof(SolveCtl));
   if (e == cudaSuccess) e = cudaMallocHost(&dk->ctl_host, sizeof(SolveCtl));
   if (e != cudaSuccess) {
@@ -361,7 +495,7 @@ int mihs_dual_sketch(const float* A, int64_t n, int64_t d, int64_t lda, int fami
   dk->g = dk->u + round_up(d, 4);
   dk->nu_prev = dk->g + dk->np;
   dk->upart = dk->nu_prev + dk->np;
-  dk->ctl = reinterpret_cast<SolveCtl*>(dk->upart + (size_t)atnu_num_splits(n) * (size_t)round_up(d, 4));
+  dk->ctl = reinterpret_cast<SolveCtl*>(dk->upart + dual_scratch_floats(n, d));
   rc = dual_sketch_into(dk, A, lda, seed, static_cast<cudaStream_t>(stream));
   if (rc) {
     cudaStreamSynchronize(static_cast<cudaStream_t>(stream));  // nothing of this handle still in flight
@@ -413,12 +547,12 @@ int mihs_gradient_dual(const float* A, int64_t n, int64_t d, int64_t lda, const 
   MIHS_ARG(lambda >= 0.0 && lambda <= (double)FLT_MAX, "mihs_gradient_dual: lambda must be in [0, FLT_MAX]");
   cudaStream_t s = static_cast<cudaStream_t>(stream);
   StreamScratch us;
-  rc = us.alloc(sizeof(float) * (size_t)round_up(d, 4) * (size_t)(1 + atnu_num_splits(n)), s);
+  rc = us.alloc(sizeof(float) * ((size_t)round_up(d, 4) + dual_scratch_floats(n, d)), s);
   if (rc) return rc;
   float* u = static_cast<float*>(us.p);
   rc = launch_atnu(A, n, d, lda, nu, u, u + round_up(d, 4), nullptr, s);
   if (rc) return rc;
-  return launch_dual_resid(A, n, d, lda, u, b, nu, (float)lambda, g, nullptr, s);
+  return launch_dual_resid(A, n, d, lda, u, b, nu, (float)lambda, g, u + round_up(d, 4), nullptr, s);
 }
 
 int mihs_dual_recover(const float* A, int64_t n, int64_t d, int64_t lda, const float* nu, float* x, void* stream) {
@@ -429,7 +563,7 @@ int mihs_dual_recover(const float* A, int64_t n, int64_t d, int64_t lda, const f
   MIHS_ARG((reinterpret_cast<uintptr_t>(x) & 15u) == 0, "mihs_dual_recover: x must be 16-byte aligned");
   cudaStream_t s = static_cast<cudaStream_t>(stream);
   StreamScratch ps;
-  const int prc = ps.alloc(sizeof(float) * (size_t)round_up(d, 4) * (size_t)atnu_num_splits(n), s);
+  const int prc = ps.alloc(sizeof(float) * dual_scratch_floats(n, d), s);
   if (prc) return prc;
   return launch_atnu(A, n, d, lda, nu, x, static_cast<float*>(ps.p), nullptr, s);
 }
@@ -538,7 +672,7 @@ int mihs_solve_dual(mihs_dual_t dk, const float* A, int64_t lda, const float* b,
   info->inner_iters_total = c.inner_total;
   info->rel_resid = c.gnorm0 > 0.f ? (double)c.gnorm / (double)c.gnorm0 : 0.0;
   info->status = c.done ? c.status : MIHS_NOT_CONVERGED;
-  if (graph_ran) count_launch(4ull * (uint64_t)(c.outer + 1));
+  if (graph_ran) count_launch((dual_plan(n, dk->d).slices > 1 ? 5ull : 4ull) * (uint64_t)(c.outer + 1));
   return info->status;
 }
 

@@ -169,6 +169,9 @@ void aab_prepare(int m, int d, int sa_type = 0);
 
 constexpr int kHistCap = 1024;
 
+// ---- dual gradient (dual.cu)
+int dual_device_error(int* code);
+
 // ---- sketches (sketch_*.cu) ------------------------------------------------
 int sketch_gaussian(const float* A, int64_t n, int64_t d, int64_t lda, int64_t m,
                     uint64_t seed, float* SA, int64_t ldsa, cudaStream_t s);
