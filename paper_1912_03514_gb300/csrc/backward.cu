@@ -48,38 +48,50 @@ __device__ __forceinline__ float dot4(const float4 a, const float4 b) {
   return fmaf(a.x, b.x, fmaf(a.y, b.y, fmaf(a.z, b.z, a.w * b.w)));
 }
 
-// Vector path: d, lda, ldda multiples of 4 and 16-byte aligned rows.  Lane
-// `l` holds columns 4(32c + l) … 4(32c + l) + 3 of chunk c < CH, CH =
-// ⌈d/128⌉; x and v live in registers (CH ≤ 4) or shared memory (CH ≥ 8:
-// held in registers they cap the CTA count per SM and, measured at 2²⁰×1024,
-// the pass ran at 0.57 of HBM bandwidth instead of 0.97).  RW rows per warp
-// iteration give each warp RW·CH independent 16-byte loads in flight.
+// Columns j … j + 3 of a vector of d elements (zero past it; any alignment).
+__device__ __forceinline__ float4 vec4(const float* v, int j, int d) {
+  return make_float4(j < d ? v[j] : 0.f, j + 1 < d ? v[j + 1] : 0.f, j + 2 < d ? v[j + 2] : 0.f,
+                     j + 3 < d ? v[j + 3] : 0.f);
+}
+
+// Rows of A are 16-byte aligned (the interface asks for that).  Lane `l` holds
+// columns 4(32c + l) … 4(32c + l) + 3 of chunk c < CH, CH = ⌈d/128⌉; x and v
+// live in registers (CH ≤ 4) or shared memory (CH ≥ 8: held in registers they
+// cap the CTA count per SM and, measured at 2²⁰×1024, the pass ran at 0.57 of
+// HBM bandwidth instead of 0.97).  RW rows per warp iteration give each warp
+// RW·CH independent 16-byte loads in flight.
+//
+// Rows of dA may start anywhere (d = 1001, say, with dense rows).  A row whose
+// start lies s floats before a 16-byte boundary is stored from there on in
+// 16-byte groups, each made of a lane's last 4 − s columns and the next lane's
+// first s (at most three shuffles per group), its first s columns by lane 0.
+// 200003×1001: 298 → 275 µs (5.8 TB/s); one element per lane throughout, or 16-byte
+// loads with consecutive 4-byte stores through shared memory (306 µs), were
+// bound by the store requests.  200003×1000, no shuffles: 264 µs.
 template <int CH, int RW>
 __global__ void __launch_bounds__(kThreads)
-    backward_rows_vec_kernel(const float* __restrict__ A, long long n, int d, long long lda,
-                             const float* __restrict__ b, const float* __restrict__ x,
-                             const float* __restrict__ v, float* __restrict__ dA, long long ldda,
-                             float* __restrict__ db) {
+    backward_rows_kernel(const float* __restrict__ A, long long n, int d, long long lda,
+                         const float* __restrict__ b, const float* __restrict__ x,
+                         const float* __restrict__ v, float* __restrict__ dA, long long ldda,
+                         float* __restrict__ db) {
   constexpr bool XS = CH >= 8;
   __shared__ float4 xs4[XS ? CH * 32 : 1], vs4[XS ? CH * 32 : 1];
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  const int d4 = d >> 2;
+  const int groups = (d + 3) >> 2, d4 = d >> 2;  // groups of four columns, and those that are full
   float4 xr[XS ? 1 : CH], vr[XS ? 1 : CH];
-  const float4* x4 = reinterpret_cast<const float4*>(x);
-  const float4* v4 = reinterpret_cast<const float4*>(v);
   const float4 z4 = make_float4(0.f, 0.f, 0.f, 0.f);
   if (XS) {
     for (int i = threadIdx.x; i < CH * 32; i += kThreads) {
-      xs4[i] = i < d4 ? x4[i] : z4;
-      vs4[i] = i < d4 ? v4[i] : z4;
+      xs4[i] = vec4(x, 4 * i, d);
+      vs4[i] = vec4(v, 4 * i, d);
     }
     __syncthreads();
   } else {
 #pragma unroll
     for (int c = 0; c < (XS ? 1 : CH); ++c) {
       const int i = c * 32 + lane;
-      xr[c] = i < d4 ? x4[i] : z4;
-      vr[c] = i < d4 ? v4[i] : z4;
+      xr[c] = vec4(x, 4 * i, d);
+      vr[c] = vec4(v, 4 * i, d);
     }
   }
   const long long nw = (long long)gridDim.x * kWarps;
@@ -88,11 +100,16 @@ __global__ void __launch_bounds__(kThreads)
 #pragma unroll
     for (int k = 0; k < RW; ++k) {
       const long long row = r0 + k;
-      const float4* Ar = reinterpret_cast<const float4*>(A + (row < n ? row : 0) * lda);
+      const float* Ar = A + (row < n ? row : 0) * lda;
 #pragma unroll
       for (int c = 0; c < CH; ++c) {
         const int i = c * 32 + lane;
-        a[k][c] = (row < n && i < d4) ? __ldg(Ar + i) : z4;
+        a[k][c] = (row < n && i < d4) ? __ldg(reinterpret_cast<const float4*>(Ar) + i) : z4;
+        if (c >= CH / 2 && row < n && i == d4 && i < groups) {  // the ragged last group
+          a[k][c].x = __ldg(Ar + 4 * i);
+          if (4 * i + 1 < d) a[k][c].y = __ldg(Ar + 4 * i + 1);
+          if (4 * i + 2 < d) a[k][c].z = __ldg(Ar + 4 * i + 2);
+        }
       }
     }
     float rr[RW], qq[RW];
@@ -122,54 +139,54 @@ __global__ void __launch_bounds__(kThreads)
       if (row >= n) break;
       if (db != nullptr && lane == 0) db[row] = qq[k];
       if (dA == nullptr) continue;
-      float4* Dr = reinterpret_cast<float4*>(dA + row * ldda);
+      float* Dr = dA + row * ldda;
+      const int s = (int)((0u - (uint32_t)(uintptr_t)Dr) >> 2) & 3;  // floats before the first boundary
+      auto grad = [&](int c) {
+        const int i = c * 32 + lane;
+        const float4 xc = XS ? xs4[i] : xr[XS ? 0 : c];
+        const float4 vc = XS ? vs4[i] : vr[XS ? 0 : c];
+        float4 o;
+        o.x = fmaf(rr[k], vc.x, -qq[k] * xc.x);
+        o.y = fmaf(rr[k], vc.y, -qq[k] * xc.y);
+        o.z = fmaf(rr[k], vc.z, -qq[k] * xc.z);
+        o.w = fmaf(rr[k], vc.w, -qq[k] * xc.w);
+        return o;
+      };
+      float4 cur = grad(0);
+      if (s > 0 && lane == 0) {
+        Dr[0] = cur.x;
+        if (s > 1 && d > 1) Dr[1] = cur.y;
+        if (s > 2 && d > 2) Dr[2] = cur.z;
+      }
 #pragma unroll
       for (int c = 0; c < CH; ++c) {
-        const int i = c * 32 + lane;
-        if (i < d4) {
-          const float4 xc = XS ? xs4[i] : xr[XS ? 0 : c];
-          const float4 vc = XS ? vs4[i] : vr[XS ? 0 : c];
-          float4 o;
-          o.x = fmaf(rr[k], vc.x, -qq[k] * xc.x);
-          o.y = fmaf(rr[k], vc.y, -qq[k] * xc.y);
-          o.z = fmaf(rr[k], vc.z, -qq[k] * xc.z);
-          o.w = fmaf(rr[k], vc.w, -qq[k] * xc.w);
-          __stcs(Dr + i, o);  // streamed: dA is written once and not re-read here
+        float4 next = z4, o = cur;
+        if (c + 1 < CH) next = grad(c + 1);
+        if (s > 0) {  // uniform across the warp
+          const int from = (lane + 1) & 31;
+          const float nx = __shfl_sync(0xffffffffu, lane == 0 ? next.x : cur.x, from);
+          if (s == 1) {
+            o = make_float4(cur.y, cur.z, cur.w, nx);
+          } else {
+            const float ny = __shfl_sync(0xffffffffu, lane == 0 ? next.y : cur.y, from);
+            if (s == 2) {
+              o = make_float4(cur.z, cur.w, nx, ny);
+            } else {
+              const float nz = __shfl_sync(0xffffffffu, lane == 0 ? next.z : cur.z, from);
+              o = make_float4(cur.w, nx, ny, nz);
+            }
+          }
         }
+        const int j = 4 * (c * 32 + lane) + s;
+        if (j + 4 <= d) {
+          __stcs(reinterpret_cast<float4*>(Dr + j), o);  // streamed: dA is not re-read here
+        } else if (j < d) {
+          Dr[j] = o.x;
+          if (j + 1 < d) Dr[j + 1] = o.y;
+          if (j + 2 < d) Dr[j + 2] = o.z;
+        }
+        cur = next;
       }
-    }
-  }
-}
-
-// Any d, lda, ldda: x and v in shared memory, two sweeps over each row (the
-// second one hits L1/L2).
-__global__ void __launch_bounds__(kThreads)
-    backward_rows_kernel(const float* __restrict__ A, long long n, int d, long long lda,
-                         const float* __restrict__ b, const float* __restrict__ x,
-                         const float* __restrict__ v, float* __restrict__ dA, long long ldda,
-                         float* __restrict__ db) {
-  __shared__ float xs[kMaxD], vs[kMaxD];
-  for (int j = threadIdx.x; j < d; j += kThreads) {
-    xs[j] = x[j];
-    vs[j] = v[j];
-  }
-  __syncthreads();
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  const long long nw = (long long)gridDim.x * kWarps;
-  for (long long row = (long long)blockIdx.x * kWarps + warp; row < n; row += nw) {
-    const float* Ar = A + row * lda;
-    float sx = 0.f, sv = 0.f;
-    for (int j = lane; j < d; j += 32) {
-      const float aij = __ldg(Ar + j);
-      sx = fmaf(aij, xs[j], sx);
-      sv = fmaf(aij, vs[j], sv);
-    }
-    const float r = (b != nullptr ? __ldg(b + row) : 0.f) - warp_sum(sx);
-    const float q = warp_sum(sv);
-    if (db != nullptr && lane == 0) db[row] = q;
-    if (dA != nullptr) {
-      float* Dr = dA + row * ldda;
-      for (int j = lane; j < d; j += 32) Dr[j] = fmaf(r, vs[j], -q * xs[j]);
     }
   }
 }
@@ -189,8 +206,6 @@ int launch_rows(K kernel, long long n, const void* const* args, cudaStream_t s) 
   return MIHS_OK;
 }
 
-bool aligned16(const void* p) { return ((uintptr_t)p & 15u) == 0; }
-
 }  // namespace
 
 int launch_backward_grads(const float* A, int64_t n, int64_t d, int64_t lda, const float* b, const float* x,
@@ -204,17 +219,14 @@ int launch_backward_grads(const float* A, int64_t n, int64_t d, int64_t lda, con
   long long n_ = n, lda_ = lda, ldda_ = dA != nullptr ? ldda : 0;
   int d_ = (int)d;
   const void* args[] = {&A, &n_, &d_, &lda_, &b, &x, &v, &dA, &ldda_, &db};
-  const bool vec = d % 4 == 0 && lda % 4 == 0 && aligned16(A) && aligned16(x) && aligned16(v) &&
-                   (dA == nullptr || (ldda % 4 == 0 && aligned16(dA)));
   const int ch = (int)((d + 127) / 128);
   timing_begin(kTimerBackward, s);
   int rc;
-  if (!vec) rc = launch_rows(backward_rows_kernel, n, args, s);
-  else if (ch <= 1) rc = launch_rows(backward_rows_vec_kernel<1, 4>, n, args, s);
-  else if (ch <= 2) rc = launch_rows(backward_rows_vec_kernel<2, 4>, n, args, s);
-  else if (ch <= 4) rc = launch_rows(backward_rows_vec_kernel<4, 2>, n, args, s);
-  else if (ch <= 8) rc = launch_rows(backward_rows_vec_kernel<8, 2>, n, args, s);
-  else rc = launch_rows(backward_rows_vec_kernel<16, 1>, n, args, s);
+  if (ch <= 1) rc = launch_rows(backward_rows_kernel<1, 4>, n, args, s);
+  else if (ch <= 2) rc = launch_rows(backward_rows_kernel<2, 4>, n, args, s);
+  else if (ch <= 4) rc = launch_rows(backward_rows_kernel<4, 2>, n, args, s);
+  else if (ch <= 8) rc = launch_rows(backward_rows_kernel<8, 2>, n, args, s);
+  else rc = launch_rows(backward_rows_kernel<16, 1>, n, args, s);
   timing_end(kTimerBackward, s);
   return rc;
 }
