@@ -5,7 +5,7 @@
 // over K = rows of A.  The tf32 MMA reads both operands K-major, while A is
 // stored with its columns contiguous, so per K-block of 32 rows:
 //   * a TMA lane loads the 32×256 tile of A (fp32) into a staging ring;
-//   * four transposer warps rewrite it K-major (one 128-byte row per column
+//   * eight transposer warps rewrite it K-major (one 128-byte row per column
 //     of A, 16-byte chunks XOR-swizzled by row mod 8 — the canonical 128-byte
 //     swizzle layout), rounding to tf32;
 //   * sixteen generator warps write the 128×32 tile of S (Philox4x32-10 counter
@@ -47,7 +47,7 @@ constexpr int TM = 128;          // sketch rows per tile (MMA M)
 constexpr int TN = 256;          // columns of A per tile (MMA N)
 constexpr int TK = 32;           // rows of A per TMA load (a tf32 stage: 4 MMAs of K = 8)
 constexpr int kGenWarps = 16;    // S generators (warps 2–17); warps 2–5 then run the epilogue
-constexpr int kTrWarps = 4;      // A transposers (warps 18–21)
+constexpr int kTrWarps = 8;      // A transposers (warps 18–25), one column of the tile per thread
 constexpr int kThreads = (2 + kGenWarps + kTrWarps) * 32;  // warp 0: MMA, warp 1: TMA
 constexpr uint32_t kSBytes = TM * TK * 4;       // one 128-row S tile: 16 KB
 constexpr uint32_t kABytes = TK * TN * 4;       // one 32-row fp32 A tile: 32 KB
@@ -356,16 +356,15 @@ gauss_tc_kernel(const __grid_constant__ CUtensorMap tmap_a, const GaussTcArgs a)
     __syncwarp();
   } else if (warp >= 2 + kGenWarps) {
     // ------------------------------------------------ A transposers: staging → K-major
-    const int tt = threadIdx.x - (2 + kGenWarps) * 32;  // 0..127: columns tt, tt + 128
+    // The stage's column is loaded and rounded before the wait for the stage: only
+    // the stores are left when its last MMAs have read it.  With the same order in
+    // the generators, S·A of 262144×1024 to 1024 rows went from 962 to 925 µs.
+    const int c = threadIdx.x - (2 + kGenWarps) * 32;  // column 0..255
     const float as = PREC == 2 ? a.ascale[0] : 1.f;
     bool stop = false;
     for (int kb = 0; kb < nkb && !stop; ++kb) {
       const int s = kb % NSTAGE;
-      if (kb >= NSTAGE && !mbar_wait(&empty[s], ((uint32_t)(kb / NSTAGE) & 1u) ^ 1u, kWaitLimitNs)) {
-        atomicExch(&g_gauss_tc_error, MIHS_ERR_TIMEOUT);
-        break;
-      }
-      unsigned char* dstA = base + (size_t)s * kStageBytes + C::SBytes;
+      uint4 v[8];  // the column's 128-byte row, in 16-byte chunks of K
 #pragma unroll
       for (int sl = 0; sl < NSLOT; ++sl) {
         const int j = kb * NSLOT + sl;
@@ -375,53 +374,43 @@ gauss_tc_kernel(const __grid_constant__ CUtensorMap tmap_a, const GaussTcArgs a)
           stop = true;
           break;
         }
-        const float* src = reinterpret_cast<const float*>(stg + (size_t)q * kABytes);  // [32 rows][256 cols]
+        const float* src = reinterpret_cast<const float*>(stg + (size_t)q * kABytes) + c;  // [32 rows][256 cols]
+        if constexpr (PREC == 2) {
+          // 16-byte chunk ch = 2·sl + hh holds K = 16ch … 16ch + 15 as e4m3
 #pragma unroll
-        for (int h = 0; h < 2; ++h) {
-          const int c = tt + 128 * h;
-          unsigned char* row = dstA + (c >> 3) * 1024 + (c & 7) * 128;
-          if constexpr (PREC == 2) {
-            // 16-byte chunk ch = 2·sl + hh holds K = 16ch … 16ch + 15 as e4m3
-#pragma unroll
-            for (int hh = 0; hh < 2; ++hh) {
-              const float* r = src + (size_t)(16 * hh) * TN + c;
-              uint4 v;
-              v.x = pack_e4m3x4(r[0 * TN] * as, r[1 * TN] * as, r[2 * TN] * as, r[3 * TN] * as);
-              v.y = pack_e4m3x4(r[4 * TN] * as, r[5 * TN] * as, r[6 * TN] * as, r[7 * TN] * as);
-              v.z = pack_e4m3x4(r[8 * TN] * as, r[9 * TN] * as, r[10 * TN] * as, r[11 * TN] * as);
-              v.w = pack_e4m3x4(r[12 * TN] * as, r[13 * TN] * as, r[14 * TN] * as, r[15 * TN] * as);
-              const int ch = 2 * sl + hh;
-              *reinterpret_cast<uint4*>(row + ((ch ^ (c & 7)) << 4)) = v;
-            }
-          } else if constexpr (PREC == 1) {
-            // 16-byte chunk ch = 4·sl + cc holds K = 8ch … 8ch + 7 as bf16
-#pragma unroll
-            for (int cc = 0; cc < 4; ++cc) {
-              const float* r = src + (size_t)(8 * cc) * TN + c;
-              uint4 v;
-              v.x = pack_bf16x2(r[0 * TN], r[1 * TN]);
-              v.y = pack_bf16x2(r[2 * TN], r[3 * TN]);
-              v.z = pack_bf16x2(r[4 * TN], r[5 * TN]);
-              v.w = pack_bf16x2(r[6 * TN], r[7 * TN]);
-              const int ch = 4 * sl + cc;
-              *reinterpret_cast<uint4*>(row + ((ch ^ (c & 7)) << 4)) = v;
-            }
-          } else {
-#pragma unroll
-            for (int ch = 0; ch < TK / 4; ++ch) {
-              uint4 v;
-              v.x = to_tf32(src[(4 * ch + 0) * TN + c]);
-              v.y = to_tf32(src[(4 * ch + 1) * TN + c]);
-              v.z = to_tf32(src[(4 * ch + 2) * TN + c]);
-              v.w = to_tf32(src[(4 * ch + 3) * TN + c]);
-              *reinterpret_cast<uint4*>(row + ((ch ^ (c & 7)) << 4)) = v;
-            }
+          for (int hh = 0; hh < 2; ++hh) {
+            const float* r = src + (size_t)(16 * hh) * TN;
+            v[2 * sl + hh] = make_uint4(
+                pack_e4m3x4(r[0 * TN] * as, r[1 * TN] * as, r[2 * TN] * as, r[3 * TN] * as),
+                pack_e4m3x4(r[4 * TN] * as, r[5 * TN] * as, r[6 * TN] * as, r[7 * TN] * as),
+                pack_e4m3x4(r[8 * TN] * as, r[9 * TN] * as, r[10 * TN] * as, r[11 * TN] * as),
+                pack_e4m3x4(r[12 * TN] * as, r[13 * TN] * as, r[14 * TN] * as, r[15 * TN] * as));
           }
+        } else if constexpr (PREC == 1) {
+          // 16-byte chunk ch = 4·sl + cc holds K = 8ch … 8ch + 7 as bf16
+#pragma unroll
+          for (int cc = 0; cc < 4; ++cc) {
+            const float* r = src + (size_t)(8 * cc) * TN;
+            v[4 * sl + cc] = make_uint4(pack_bf16x2(r[0 * TN], r[1 * TN]), pack_bf16x2(r[2 * TN], r[3 * TN]),
+                                        pack_bf16x2(r[4 * TN], r[5 * TN]), pack_bf16x2(r[6 * TN], r[7 * TN]));
+          }
+        } else {
+#pragma unroll
+          for (int ch = 0; ch < TK / 4; ++ch)
+            v[ch] = make_uint4(to_tf32(src[(4 * ch + 0) * TN]), to_tf32(src[(4 * ch + 1) * TN]),
+                               to_tf32(src[(4 * ch + 2) * TN]), to_tf32(src[(4 * ch + 3) * TN]));
         }
         __syncwarp();
         if (lane == 0) mbar_arrive(&stg_empty[q]);  // this warp's reads of the slot are done
       }
       if (stop) break;
+      if (kb >= NSTAGE && !mbar_wait(&empty[s], ((uint32_t)(kb / NSTAGE) & 1u) ^ 1u, kWaitLimitNs)) {
+        atomicExch(&g_gauss_tc_error, MIHS_ERR_TIMEOUT);
+        break;
+      }
+      unsigned char* row = base + (size_t)s * kStageBytes + C::SBytes + (c >> 3) * 1024 + (c & 7) * 128;
+#pragma unroll
+      for (int ch = 0; ch < 8; ++ch) *reinterpret_cast<uint4*>(row + ((ch ^ (c & 7)) << 4)) = v[ch];
       fence_async_shared();  // generic-proxy writes → visible to the tensor core
       __syncwarp();
       if (lane == 0) mbar_arrive(&full[s]);
@@ -434,22 +423,18 @@ gauss_tc_kernel(const __grid_constant__ CUtensorMap tmap_a, const GaussTcArgs a)
     const int g = threadIdx.x - 64;
     const int nitems = (g_hi - g_lo) * 8;
     const uint32_t slice_off = (uint32_t)g_lo * 128u, slice_bytes = (uint32_t)(g_hi - g_lo) * 128u;
+    // The stage's entries are generated before the wait for the stage (a few
+    // hundred cycles that used to lie between the last MMA on it and the next).
+    constexpr int NI = MROWS * 8 / (kGenWarps * 32);  // items per thread with one block per cluster
     for (int kb = 0; kb < nkb; ++kb) {
       const int s = kb % NSTAGE;
       const uint32_t ph = (uint32_t)(kb / NSTAGE) & 1u;
-      if (kb >= NSTAGE) {
-        // One thread waits (bounded) and every generator takes its decision, so
-        // that all of them reach the same named barriers.
-        if (g == 0) *gen_abort = mbar_wait(&empty[s], ph ^ 1u, kWaitLimitNs) ? 0u : 1u;
-        named_sync(1, kGenWarps * 32);
-        if (*gen_abort) {
-          if (g == 0) atomicExch(&g_gauss_tc_error, MIHS_ERR_TIMEOUT);
-          break;
-        }
-      }
-      unsigned char* sS = base + (size_t)s * kStageBytes;
       const int kbase = kb0 + kb * KT;
-      for (int e = g; e < nitems; e += kGenWarps * 32) {
+      uint4 items[NI];
+#pragma unroll
+      for (int i = 0; i < NI; ++i) {
+        const int e = g + i * kGenWarps * 32;
+        if (e >= nitems) break;
         const int gt = g_lo + (e >> 3), c = e & 7;
         const int gi = i0 + gt;
         uint4 out = make_uint4(0u, 0u, 0u, 0u);
@@ -507,7 +492,25 @@ gauss_tc_kernel(const __grid_constant__ CUtensorMap tmap_a, const GaussTcArgs a)
                              j0 + 2 < kb1 ? to_tf32(zb.x) : 0u, j0 + 3 < kb1 ? to_tf32(zb.y) : 0u);
           }
         }
-        *reinterpret_cast<uint4*>(sS + (size_t)gt * 128 + ((c ^ (gt & 7)) << 4)) = out;
+        items[i] = out;
+      }
+      if (kb >= NSTAGE) {
+        // One thread waits (bounded) and every generator takes its decision, so
+        // that all of them reach the same named barriers.
+        if (g == 0) *gen_abort = mbar_wait(&empty[s], ph ^ 1u, kWaitLimitNs) ? 0u : 1u;
+        named_sync(1, kGenWarps * 32);
+        if (*gen_abort) {
+          if (g == 0) atomicExch(&g_gauss_tc_error, MIHS_ERR_TIMEOUT);
+          break;
+        }
+      }
+      unsigned char* sS = base + (size_t)s * kStageBytes;
+#pragma unroll
+      for (int i = 0; i < NI; ++i) {
+        const int e = g + i * kGenWarps * 32;
+        if (e >= nitems) break;
+        const int gt = g_lo + (e >> 3), c = e & 7;
+        *reinterpret_cast<uint4*>(sS + (size_t)gt * 128 + ((c ^ (gt & 7)) << 4)) = items[i];
       }
       fence_async_shared();            // the slice → visible to the async proxy (MMA, bulk copies)
       named_sync(1, kGenWarps * 32);   // every generator has written its part
