@@ -36,6 +36,24 @@ def test_path_gradient_is_exact(n, d, nl):
     assert mihs.device_status() == 0
 
 
+# the last width of each form of the path kernel and the first of the next, with the most iterates that take half of
+# it and the first that take both; rows that fill the rings several times, and a last stage of 1 to 3 rows
+@pytest.mark.parametrize("n,d,nl", [(60001, 128, 8), (60002, 129, 9), (30003, 256, 9), (30000, 257, 8),
+                                    (30001, 512, 8), (30002, 513, 9), (15003, 768, 8), (15000, 769, 8),
+                                    (15001, 1024, 8), (2, 768, 16)])
+def test_path_gradient_widths_are_exact(n, d, nl):
+    A, An = _matrix(n, d, n + d, -1, 1)
+    b = W.randint_matrix((n,), 3, -9, 9)
+    X = W.randint_matrix((nl, d), 4, -1, 1)
+    lams = [float(l % 3) for l in range(nl)]
+    G = mihs.gradient_path(A, b.to(DEV), X.to(DEV), lams).cpu().double().numpy()
+    Xn = X.double().numpy()
+    ref = (b.double().numpy()[:, None] - An @ Xn.T).T @ An - np.array(lams)[:, None] * Xn
+    assert np.abs(ref).max() < 2 ** 24
+    assert np.array_equal(G, ref)
+    assert mihs.device_status() == 0
+
+
 # n, d: one group of columns and less, each width of the kernel with and without 16-byte rows of dA, staged in two
 # halves past 1024 columns, the last row's last group
 @pytest.mark.parametrize("n,d", [(1, 1), (5, 3), (64, 4), (33, 127), (100, 129), (257, 255), (300, 512), (301, 510),
