@@ -20,7 +20,9 @@
 // at 1600 × 1024: 196 → 123 µs; what remains per pass is two trips store → L2
 // → poll → load (≈ 1.6 K cycles each) and the block's ≈ 2.5 K cycles of work.
 // Tags grow from launch to launch (`epoch`), so the words need no clearing
-// between them.  Every sum over blocks has a fixed order: all blocks compute
+// between the launches of a solve; before it they are cleared.  In a solve of
+// more than 2²⁰ steps the tags wrap: a word that any of those steps wrote then
+// holds a newer tag, so none passes for the new one.  Every sum over blocks has a fixed order: all blocks compute
 // the same scalars and take the same branches.
 //
 // A word is overwritten only after everyone who polls it has answered with
@@ -499,7 +501,8 @@ __global__ void __launch_bounds__(kThreads, 1) aab_gridreg_kernel(const GridRegP
     }
     failed = __syncthreads_or(!ok) != 0;
   }
-  if (tid == 0 && (failed || blk == 0)) atomicMax(P.epoch, base + kEpochStep);
+  // (all that write it write the same; it wraps at 2³²)
+  if (tid == 0 && (failed || blk == 0)) atomicExch(P.epoch, base + kEpochStep);
   if (failed) {
     if (tid == 0) {
       atomicExch(&g_aab_gridreg_error, MIHS_ERR_TIMEOUT);

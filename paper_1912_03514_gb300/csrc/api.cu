@@ -249,7 +249,6 @@ struct mihs_sketch_s {
   // (P_path × 16 × dp), G and X⁻ (16 × dp each), 16 control blocks and the
   // path's stop counter / flag.
   void* aab_grid_ws = nullptr;   // global scratch of the single-λ grid AAb kernel (first solve that needs it)
-  int aab_grid_ws_type = 0, aab_grid_ws_blocks = 0;  // the launches it was prepared for
   int aab_form = MIHS_AAB_AUTO;  // form of AAb_Solver in single-λ solves (mihs_sketch_set_aab)
   int aab_grid_blocks = 0;
   float* path_partials = nullptr;
@@ -299,13 +298,11 @@ void set_sa(AabLaunch& a, const mihs_sketch_s* sk) {
 
 // The grid form of AAb_Solver (SA too large for one cluster's shared memory,
 // or asked for by mihs_sketch_set_aab) needs global scratch: the handle's,
-// allocated on first use; its barrier word is zeroed on the solve's stream
-// before every solve.
+// allocated on first use and prepared on the solve's stream before every solve.
 int use_grid_ws(mihs_sketch_s* sk, AabLaunch& a, cudaStream_t s) {
   a.aab_form = sk->aab_form;
   a.grid_blocks = sk->aab_grid_blocks;
   if (!aab_grid_wanted(a.m, a.d, a.sa_type, a.aab_form)) return MIHS_OK;
-  bool fresh = false;
   if (sk->aab_grid_ws == nullptr) {
     const size_t bytes = aab_grid_ws_bytes(a.d);
     cudaError_t e = cudaMalloc(&sk->aab_grid_ws, bytes);
@@ -314,16 +311,9 @@ int use_grid_ws(mihs_sketch_s* sk, AabLaunch& a, cudaStream_t s) {
       set_error("AAb grid scratch: cudaMalloc(%zu): %s", bytes, cudaGetErrorString(e));
       return e == cudaErrorMemoryAllocation ? MIHS_ERR_OOM : MIHS_ERR_CUDA;
     }
-    fresh = true;
   }
-  if (fresh || sk->aab_grid_ws_type != a.sa_type || sk->aab_grid_ws_blocks != a.grid_blocks) {
-    const int rc = aab_grid_ws_init(sk->aab_grid_ws, a.d, s);
-    if (rc) return rc;
-    sk->aab_grid_ws_type = a.sa_type;
-    sk->aab_grid_ws_blocks = a.grid_blocks;
-  } else {
-    MIHS_CUDA_TRY(cudaMemsetAsync(sk->aab_grid_ws, 0, kAabGridBarBytes, s));
-  }
+  const int rc = aab_grid_ws_init(sk->aab_grid_ws, a.d, s);
+  if (rc) return rc;
   a.grid_ws = sk->aab_grid_ws;
   return MIHS_OK;
 }

@@ -627,10 +627,9 @@ int mihs_solve_dual(mihs_dual_t dk, const float* A, int64_t lda, const float* b,
         set_error("mihs_solve_dual: cudaMalloc(%zu): %s", bytes, cudaGetErrorString(e));
         return e == cudaErrorMemoryAllocation ? MIHS_ERR_OOM : MIHS_ERR_CUDA;
       }
-      rc = aab_grid_ws_init(dk->grid_ws, a.d, s);
-      if (rc) return rc;
     }
-    MIHS_CUDA_TRY(cudaMemsetAsync(dk->grid_ws, 0, kAabGridBarBytes, s));
+    rc = aab_grid_ws_init(dk->grid_ws, a.d, s);
+    if (rc) return rc;
     a.grid_ws = dk->grid_ws;
   }
   const mihs_dual_s::Key key = {A, lda, b, nu, lambda, alpha, beta, a.eps, a.max_passes};

@@ -141,9 +141,8 @@ int launch_aab(const AabLaunch& a, cudaStream_t s);
 constexpr size_t kAabGridBarBytes = 256;
 size_t aab_grid_ws_bytes(int d);
 int launch_aab_grid(const AabLaunch& a, void* ws, cudaStream_t s);
-// Makes freshly allocated scratch usable (and scratch whose next launches take
-// another block count or storage type than the last): clears the barrier word
-// and the tagged words of the register form (aab_grid_reg.cu).
+// Prepares scratch for a solve, whatever it held: clears the barrier word and
+// the tagged words of the register form (aab_grid_reg.cu), 2.8 MB at d = 2048.
 int aab_grid_ws_init(void* ws, int d, cudaStream_t s);
 // The register form of the grid, on its part of the scratch; UNSUPPORTED
 // (nothing launched) when `blocks` blocks do not hold SA in registers.
