@@ -207,10 +207,10 @@ int mihs_gradient_noalloc(const float* A, int64_t n, int64_t d, int64_t lda,
  *   passes: optional DEVICE int* receiving the number of loop passes.
  * Any ldsa ≥ d is accepted when SA fits in the cluster's shared memory
  * (m·d ≲ 800K); larger SA must have 16-byte aligned rows (ldsa % 4 == 0).
- * Runs as one thread-block cluster with SA in its shared memory; an SA too
- * large for that runs as one cooperative grid of up to one block per SM with
- * SA spread over their shared memory, whose scratch (one d-vector per SM,
- * about 1.2 MB at d = 2048) comes from the stream-ordered pool and is freed
+ * Runs as one thread-block cluster with SA in its registers or shared memory;
+ * an SA too large for that runs as one cooperative grid of up to one block
+ * per SM with SA spread over theirs, whose scratch (two d-vectors per SM and
+ * a few more, 4 MB at d = 2048) comes from the stream-ordered pool and is freed
  * on the same stream (the environment variable MIHS_AAB_FORM=cluster keeps
  * one cluster reading SA from L2 instead).  Grid-form calls on different
  * streams should not overlap: two grids that wait for each other's blocks
@@ -314,9 +314,9 @@ int mihs_sketch_set_precision(mihs_sketch_t sk, int sa_prec, void* stream);
 
 /* Form of the inner solver (AAb_Solver, Algorithm 5) in a handle's solves
  * (mihs_solve, mihs_solve_refined, mihs_backward*):
- *   MIHS_AAB_AUTO     one thread-block cluster holding SA in its distributed
- *                     shared memory when it fits, else one cooperative grid
- *                     holding SA in the shared memory of up to every SM;
+ *   MIHS_AAB_AUTO     one thread-block cluster holding SA in its registers or
+ *                     distributed shared memory when it fits, else one
+ *                     cooperative grid holding SA in those of up to every SM;
  *   MIHS_AAB_CLUSTER  always one cluster (SA read from L2 when it does not
  *                     fit);
  *   MIHS_AAB_GRID     one cooperative grid of `grid_blocks` blocks (0: one per

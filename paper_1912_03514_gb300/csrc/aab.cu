@@ -20,7 +20,7 @@
 // work, negligible next to the O(md/CL) products).
 //
 // That is the form for sketches whose rows fit the shared memory of a cluster
-// but not its registers; aab_reg.cuh, which is faster (66 against 141 µs for 30
+// but not its registers; aab_reg.cuh, which is faster (68 against 141 µs for 30
 // passes at 588 × 1024), takes all that do.  When SA is too large for
 // the shared memory of 16 blocks, launch_aab hands a single-λ solve that has
 // scratch to the grid form (aab_grid.cu); otherwise the cluster's blocks

@@ -20,7 +20,7 @@
 //     and the forward substitution are computed; the dots start on θv before θ
 //     is known, and θ² is one more of them, taken by every warp from the whole
 //     vector rather than exchanged.
-// 588 × 1024, 30 passes: 141 → 66 µs, 700 × 256: 177 → 50 µs (the form with SA
+// 588 × 1024, 30 passes: 141 → 68 µs, 700 × 256: 177 → 52 µs (the form with SA
 // in shared memory swept it twice per pass and crossed two cluster barriers
 // and two remote-load round trips).
 // Every sum has a fixed order and every block computes the same scalars from
