@@ -167,7 +167,8 @@ int mihs_sketch_gaussian_fp8(const float* A, int64_t n, int64_t d, int64_t lda,
 /* Gradient step of Algorithm 1: g = Aᵀ(b − Ax) − λx, reading A once.
  *   b (n), x (d) inputs; g (d) output.  0 ≤ λ ≤ FLT_MAX (fp32 arithmetic).
  * Allocates stream-ordered scratch for the split-K partial sums (one d-vector
- * per thread block) and frees it on the same stream.  The reduction order is
+ * per thread block; none for small matrices, which take one launch without)
+ * and frees it on the same stream.  The reduction order is
  * fixed, so repeated calls give bit-identical g.
  * Errors: INVALID_ARG, CUDA, OOM. */
 int mihs_gradient(const float* A, int64_t n, int64_t d, int64_t lda,

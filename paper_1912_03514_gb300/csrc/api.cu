@@ -614,6 +614,8 @@ int mihs_gradient(const float* A, int64_t n, int64_t d, int64_t lda, const float
   MIHS_ARG(b != nullptr && x != nullptr && g != nullptr, "mihs_gradient: null vector");
   MIHS_ARG(lambda >= 0.0 && lambda <= (double)FLT_MAX, "mihs_gradient: lambda must be in [0, FLT_MAX]");
   cudaStream_t s = static_cast<cudaStream_t>(stream);
+  rc = launch_gradient_small(A, n, d, lda, b, x, (float)lambda, g, s);
+  if (rc != MIHS_ERR_UNSUPPORTED) return rc;
   const int P = apass_num_partials(n, d);
   StreamScratch scratch;
   rc = scratch.alloc(sizeof(float) * (size_t)P * apass_dpad(d), s);

@@ -85,10 +85,12 @@ extern "C" int mihs_gradient_noalloc(const float* A, int64_t n, int64_t d, int64
               "more than the fixed %zu", need, P, (long long)apass_dpad(d), kNoAllocFloats);
     return MIHS_ERR_UNSUPPORTED;
   }
-  float* scratch = nullptr;
-  int rc = scratch_for_current_device(&scratch);
-  if (rc) return rc;
   cudaStream_t s = static_cast<cudaStream_t>(stream);
+  int rc = launch_gradient_small(A, n, d, lda, b, x, (float)lambda, g, s);
+  if (rc != MIHS_ERR_UNSUPPORTED) return rc;
+  float* scratch = nullptr;
+  rc = scratch_for_current_device(&scratch);
+  if (rc) return rc;
   rc = launch_apass_partial(A, n, d, lda, b, x, scratch, nullptr, s);
   if (rc) return rc;
   return launch_apass_finalize(scratch, P, d, x, (float)lambda, g, nullptr, s);

@@ -26,6 +26,10 @@ int launch_apass_partial(const float* A, int64_t n, int64_t d, int64_t lda,
                          const double* xref = nullptr, int timer = 0 /* kTimerApass */);
 // Reads and clears the library-wide device error word (synchronises).
 int apass_device_error(int* code);
+// g = Aᵀ(b − Ax) − λx in one launch without scratch (gradient_small.cu);
+// UNSUPPORTED (nothing launched) for matrices that are not small.
+int launch_gradient_small(const float* A, int64_t n, int64_t d, int64_t lda, const float* b, const float* x,
+                          float lambda, float* g, cudaStream_t s);
 // g[j] = rhs[j] + Σ_p partials[p][j] − λ·x[j] in a fixed order (rhs may be null).
 int launch_apass_finalize(const float* partials, int P, int64_t d,
                           const float* x, float lambda, float* g,

@@ -54,6 +54,24 @@ def test_path_gradient_widths_are_exact(n, d, nl):
     assert mihs.device_status() == 0
 
 
+# one row and less than a warp's of them, each width of the one-launch form, rows that end inside a group of eight, the
+# largest matrix it takes and the first it does not; the result over x where x has its shape
+@pytest.mark.parametrize("n,d", [(1, 1), (15, 3), (16, 128), (300, 129), (4095, 256), (4099, 257), (1000, 509),
+                                 (4096, 512), (4097, 512), (16384, 128), (16385, 128), (8191, 255)])
+def test_small_gradient_is_exact(n, d):
+    A, An = _matrix(n, d, 7 * n + d, -1, 1)
+    b, x = W.randint_matrix((n,), 11, -9, 9), W.randint_matrix((d,), 12, -2, 2)
+    bn, xn = b.double().numpy(), x.double().numpy()
+    ref = An.T @ (bn - An @ xn) - 3.0 * xn
+    assert np.abs(ref).max() < 2 ** 24
+    off = torch.zeros(d + 1, device=DEV)  # x not 16-byte aligned
+    off[1:] = x.to(DEV)
+    bd = b.to(DEV)
+    assert np.array_equal(mihs.gradient(A, bd, off[1:], 3.0).cpu().double().numpy(), ref)
+    mihs.gradient(A, bd, off[1:], 3.0, g=off[1:])
+    assert np.array_equal(off[1:].cpu().double().numpy(), ref)
+
+
 # n, d: one group of columns and less, each width of the kernel with and without 16-byte rows of dA, staged in two
 # halves past 1024 columns, the last row's last group
 @pytest.mark.parametrize("n,d", [(1, 1), (5, 3), (64, 4), (33, 127), (100, 129), (257, 255), (300, 512), (301, 510),
