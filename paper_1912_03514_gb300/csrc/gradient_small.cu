@@ -24,9 +24,12 @@ constexpr int kCluster = 16;
 constexpr int kWarps = 16;
 constexpr int kThreads = kWarps * 32;
 constexpr int kSmallMaxD = 512;
-// 16 SMs draw about a quarter of the HBM bandwidth that all of them do: up to
-// 8 MB the launch saved is worth more.
-constexpr int64_t kSmallElems = 2 << 20;
+// n × the columns that the lanes cover (256, or 512 from d = 257).  16 SMs draw a
+// quarter of the bandwidth that all of them do, and the cost goes by rows as
+// much as by bytes.  Up to this line the host still bounds the call: 14.5 µs at
+// 8192×512, 16384×256 and 16384×128, where the pass over all SMs takes 20–22;
+// twice as far it is 23, 25 and 23 against 20.
+constexpr int64_t kSmallElems = 4 << 20;
 
 __device__ __forceinline__ uint32_t mapa_u32(uint32_t saddr, uint32_t rank) {
   uint32_t r;
@@ -158,7 +161,7 @@ SmallKernel probe(const void* fn) {
 
 int launch_gradient_small(const float* A, int64_t n, int64_t d, int64_t lda, const float* b, const float* x,
                           float lambda, float* g, cudaStream_t s) {
-  if (d > kSmallMaxD || n * apass_dpad(d) > kSmallElems) return MIHS_ERR_UNSUPPORTED;
+  if (d > kSmallMaxD || n * (d <= 256 ? 256 : 512) > kSmallElems) return MIHS_ERR_UNSUPPORTED;
   static const SmallKernel k1 = probe((const void*)&gradient_small_kernel<1, 8>);
   static const SmallKernel k2 = probe((const void*)&gradient_small_kernel<2, 8>);
   static const SmallKernel k4 = probe((const void*)&gradient_small_kernel<4, 4>);

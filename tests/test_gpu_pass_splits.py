@@ -57,7 +57,8 @@ def test_path_gradient_widths_are_exact(n, d, nl):
 # one row and less than a warp's of them, each width of the one-launch form, rows that end inside a group of eight, the
 # largest matrix it takes and the first it does not; the result over x where x has its shape
 @pytest.mark.parametrize("n,d", [(1, 1), (15, 3), (16, 128), (300, 129), (4095, 256), (4099, 257), (1000, 509),
-                                 (4096, 512), (4097, 512), (16384, 128), (16385, 128), (8191, 255)])
+                                 (4096, 512), (8192, 512), (8193, 512), (16384, 128), (16385, 128),
+                                 (16383, 256), (16385, 255)])
 def test_small_gradient_is_exact(n, d):
     A, An = _matrix(n, d, 7 * n + d, -1, 1)
     b, x = W.randint_matrix((n,), 11, -9, 9), W.randint_matrix((d,), 12, -2, 2)
