@@ -100,8 +100,8 @@ gradient_small_kernel(const float* __restrict__ A, int n, int d, long long lda, 
       for (int r = 0; r < RW; ++r) s[r] += __shfl_xor_sync(0xffffffffu, s[r], o);
 #pragma unroll
     for (int r = 0; r < RW; ++r) {
-      // (a row past the block's is zero, and so is its residual)
-      const float res = bi[r] - s[r];
+      // (a row past the block's is zero; its product with an infinite x is not)
+      const float res = i0 + r * kWarps < r1 ? bi[r] - s[r] : 0.f;
 #pragma unroll
       for (int c = 0; c < CH; ++c) {
         acc[c].x = fmaf(res, a[r][c].x, acc[c].x);

@@ -73,6 +73,16 @@ def test_small_gradient_is_exact(n, d):
     assert np.array_equal(off[1:].cpu().double().numpy(), ref)
 
 
+# an infinite x: the rows of a block's last group that do not exist add nothing
+@pytest.mark.parametrize("n,d", [(5, 3), (70, 130), (300, 260)])
+def test_small_gradient_of_an_infinite_iterate(n, d):
+    x = torch.zeros(d)
+    x[1] = float("inf")
+    A, _ = _matrix(n, d, 1, 1, 1)
+    g = mihs.gradient(A, torch.zeros(n, device=DEV), x.to(DEV), 1.0)
+    assert torch.equal(g.cpu(), torch.full((d,), -float("inf")))
+
+
 # n, d: one group of columns and less, each width of the kernel with and without 16-byte rows of dA, staged in two
 # halves past 1024 columns, the last row's last group
 @pytest.mark.parametrize("n,d", [(1, 1), (5, 3), (64, 4), (33, 127), (100, 129), (257, 255), (300, 512), (301, 510),
