@@ -229,12 +229,13 @@ apass_finalize_kernel(const float* __restrict__ partials, int P, int d, int dpad
 struct ApassKernel {
   const void* fn;
   int rows_per_stage;
+  int x_floats;  // shared memory for x: all columns that the kernel covers, none when x is in registers
 };
 
 template <int CH, int RW>
 ApassKernel make_kernel() {
   return ApassKernel{reinterpret_cast<const void*>(&apass_partial_kernel<CH, RW>),
-                     kConsumerWarps * RW};
+                     kConsumerWarps * RW, CH > 8 ? CH * 128 : 0};
 }
 
 ApassKernel pick(int64_t d) {
@@ -276,7 +277,7 @@ int launch_apass_partial(const float* A, int64_t n, int64_t d, int64_t lda, cons
   int stages = (int)(kRingBudget / stage_bytes);
   stages = stages < 2 ? 2 : (stages > 8 ? 8 : stages);
   const size_t smem = (size_t)stages * stage_bytes + 2 * sizeof(uint64_t) * stages +
-                      (size_t)((d + 127) / 128) * 128 * sizeof(float);
+                      (size_t)k.x_floats * sizeof(float);
   MIHS_CUDA_TRY(cudaFuncSetAttribute(k.fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
   int n32 = (int)n, d32 = (int)d, dp32 = (int)dpad;
   long long lda64 = lda;

@@ -73,6 +73,21 @@ def test_small_gradient_is_exact(n, d):
     assert np.array_equal(off[1:].cpu().double().numpy(), ref)
 
 
+# rows wider than 1024, whose x is in shared memory for all columns that the kernel covers (1536 or 2048): each number of
+# 128-column groups from the first to the last of either, the widths on both sides of a step
+@pytest.mark.parametrize("n,d", [(2000, 1025), (2003, 1152), (1999, 1153), (2001, 1280), (700, 1281), (2005, 1408),
+                                 (2000, 1409), (2002, 1536), (1997, 1537), (2003, 1664), (2001, 1665), (5, 1792),
+                                 (2004, 1793), (2001, 1920), (2002, 1921), (2003, 2047)])
+def test_wide_gradient_is_exact(n, d):
+    A, An = _matrix(n, d, n + d, -1, 1)
+    b, x = W.randint_matrix((n,), 11, -9, 9), W.randint_matrix((d,), 12, -1, 1)
+    bn, xn = b.double().numpy(), x.double().numpy()
+    ref = An.T @ (bn - An @ xn) - 3.0 * xn
+    assert np.abs(ref).max() < 2 ** 24
+    assert np.array_equal(mihs.gradient(A, b.to(DEV), x.to(DEV), 3.0).cpu().double().numpy(), ref)
+    assert mihs.device_status() == 0
+
+
 # an infinite x: the rows of a block's last group that do not exist add nothing
 @pytest.mark.parametrize("n,d", [(5, 3), (70, 130), (300, 260)])
 def test_small_gradient_of_an_infinite_iterate(n, d):
