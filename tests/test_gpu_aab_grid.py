@@ -235,6 +235,20 @@ def test_handle_aab_form_reaches_the_solution(shape):
     assert mihs.device_status() == 0
 
 
+@pytest.mark.parametrize("blocks", [0, 24])
+def test_grid_solve_that_stops_at_once(blocks):
+    """A tolerance of 2 stops the first step, which is also the one that learns ‖g(0)‖: block 0 writes the control
+    block only when every block has taken its decision from it."""
+    p = W.problem_small()
+    A, b = p.A.to(DEV), p.b.to(DEV)
+    with mihs.Sketch(A, "gaussian", p.m, seed=13) as sk:
+        sk.set_aab("grid", blocks)
+        for _ in range(50):
+            x, info = sk.solve(A, b, p.lam, p.sd, tol=2.0, max_outer=20)
+            assert info.converged and info.outer_iters == 0 and not torch.any(x), info
+    assert mihs.device_status() == 0
+
+
 def test_handle_aab_form_arguments():
     p = W.problem_small()
     with mihs.Sketch(p.A.to(DEV), "gaussian", p.m, seed=13) as sk:
