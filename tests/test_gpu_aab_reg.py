@@ -1,12 +1,15 @@
 """AAb_Solver with SA in registers, at the edges of its splits, against the oracle."""
+import ctypes
 import math
+import os
+import subprocess
 
 import numpy as np
 import pytest
 import torch
 
 from oracle import mihs_oracle as o
-from paper_1912_03514_gb300 import mihs
+from paper_1912_03514_gb300 import _build, mihs
 from paper_1912_03514_gb300 import workloads as W
 from tests._tol import U32
 from tests.test_gpu_parity import _fp32_amplification, _sa_case
@@ -55,3 +58,45 @@ def test_register_form_decodes_quantised(m, d, prec):
     a = mihs.aab_solve_q(q, prec, sc, d, g.to(DEV), 0.3, eps_sub=0.0, max_inner=9)
     b = mihs.aab_solve(dec.contiguous(), g.to(DEV), 0.3, eps_sub=0.0, max_inner=9)
     assert torch.equal(a, b)
+
+
+NORM_KERNEL = """
+#include "aab_kernel.cuh"
+__global__ void norms(const float* x, float* nrm, float* inv, int n) {
+  const int i = blockIdx.x * blockDim.x + threadIdx.x;
+  if (i < n) mihs::aabk::norm_of(x[i], nrm[i], inv[i]);
+}
+extern "C" int run(const float* x, float* nrm, float* inv, int n) {
+  norms<<<(n + 255) / 256, 256>>>(x, nrm, inv, n);
+  return (int)cudaDeviceSynchronize();
+}
+"""
+
+
+def test_norm_and_reciprocal_are_rounded_like_ieee(tmp_path):
+    """Every exponent of fp32, both lines between the two ways of computing them, zero, infinity and NaN: within half
+    a unit in the last place and a thousandth of the root, and of the rounded root's reciprocal."""
+    src, so = tmp_path / "norms.cu", tmp_path / "norms.so"
+    src.write_text(NORM_KERNEL)
+    subprocess.run([_build.nvcc(), *_build.ARCH, *_build.FLAGS, "-I", _build.CSRC, "-shared", str(src), "-o", str(so)],
+                   check=True)
+    rng = np.random.default_rng(5)
+    bits = rng.integers(1, 0x7F800000, 1 << 21, dtype=np.int64).astype(np.uint32)  # all exponents alike
+    line = np.array([1e-30, 3e38], np.float32).view(np.uint32)
+    near = (line[:, None].astype(np.int64) + np.arange(-300, 301)).reshape(-1).astype(np.uint32)
+    four = (np.float32(1).view(np.uint32) + np.arange(1 << 20, dtype=np.int64) * 16).astype(np.uint32)  # [1, 4)
+    x = np.concatenate([bits, near, four, np.array([0, 1, 0x7F7FFFFF], np.uint32)]).view(np.float32)
+    xd = torch.from_numpy(np.concatenate([x, np.array([np.inf, np.nan], np.float32)])).to(DEV)
+    nd, vd = torch.empty_like(xd), torch.empty_like(xd)
+    lib = ctypes.CDLL(os.fspath(so))
+    p = ctypes.c_void_p
+    assert lib.run(p(xd.data_ptr()), p(nd.data_ptr()), p(vd.data_ptr()), ctypes.c_int(xd.numel())) == 0
+    nrm, inv = nd.cpu().numpy(), vd.cpu().numpy()
+    assert np.isposinf(nrm[-2]) and inv[-2] == 0 and np.isnan(nrm[-1]) and np.isnan(inv[-1])
+    assert nrm[-5] == 0 and np.isposinf(inv[-5])
+    nrm, inv = nrm[:-2], inv[:-2]
+    on = x > 0
+    half = 0.5 + 2.0 ** -10
+    assert np.all(np.abs(nrm - np.sqrt(x.astype(np.float64))) <= half * np.spacing(nrm))
+    want = 1.0 / nrm[on].astype(np.float64)
+    assert np.all(np.abs(inv[on] - want) <= half * np.spacing(want.astype(np.float32)))
