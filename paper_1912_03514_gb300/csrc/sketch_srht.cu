@@ -17,19 +17,23 @@
 // SM, so no shared-memory ring and no producer are needed), transforms the
 // high five bits of the row index, passes through shared memory once,
 // transforms the low five, and adds the signed sampled rows into accumulators
-// held in registers (up to kAccMax·32 samples per block; more samples take
-// more blocks over the same, L2-resident, rows).  All additions are packed
-// pairs (f32x2: half the issue slots of scalar ones).
+// held in registers (kAccMax·32 samples per block) and, past those, in shared
+// memory (kExtra more).  Only what exceeds both takes a second block over the
+// same, L2-resident, rows.  All additions are packed pairs (f32x2: half the issue
+// slots of scalar ones).
 //
 // What bounds it: the shared-memory and load pipe (3500 wavefronts per unit, a
 // third of them the 64-byte segments of the loads) is busy 58 % of the time on
 // an SM with two blocks, the FP32 pipe 30 %, HBM 37 %; the phases of a unit
 // follow one another, and only the other block of the SM fills the gaps.  The
 // next unit's loads are issued before the samples are gathered (307 → 295 µs),
-// and slices have one range more where blocks are left (→ 274 µs).
-// 200000×1000, m = 600: 387 → 274 µs a sketch.  The form it replaces (512 × 32
+// and slices have one range more where blocks are left (→ 267 µs).
+// 200000×1000, m = 600: 390 → 267 µs a sketch.  The form it replaces (512 × 32
 // units through a TMA ring, one column per lane, accumulators in shared
-// memory) executed 2.3 times the instructions (214 M against 95 M).
+// memory) executed 2.3 times the instructions (214 M against 95 M).  With more
+// samples, that form → this one: 262144×1024 to 641 rows 506 → 334 µs, 1000
+// 864 → 394, 1240 974 → 545, 1281 (two blocks) 990 → 718, 3076 3038 → 1480; a
+// block of its own for each 640 samples took 654 µs at 641 and 700 rows.
 #include <cmath>
 
 #include "internal.h"
@@ -43,7 +47,12 @@ constexpr int kThreads = 256;   // 8 lanes per row × 32 row classes
 constexpr int kB = 1024;        // rows per unit: 32 × 32
 constexpr int kLB = 10;
 constexpr int kAccMax = 20;     // sampled rows per thread: 40 of the 128 registers of two blocks per SM
-constexpr int kMaxM = 12672;    // accepted m for n ≥ 1024
+// More sampled rows whose sums a block keeps in shared memory: at 72 bytes each as
+// many as leave room for two blocks per SM.
+constexpr int kExtra = 600;
+// Accepted m for n ≥ 1024, the interface's own limit from its first form on: six
+// times the widest matrix, past any sketch in use (m ≤ n bounds it below that).
+constexpr int kMaxM = 12672;
 // Row r of a unit starts at float 16·r + 16·(r/32): the 64-byte shift every 32
 // rows keeps the second stage's reads (rows 32 apart) free of bank conflicts.
 constexpr int kYFloats = kB * kW + (kB / 32) * kW;
@@ -76,11 +85,11 @@ __device__ __forceinline__ P2 p2_sub(P2 a, P2 b) {
   asm("sub.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
   return d;
 }
-// (x, y) with both signs flipped when bit 31 of f is set.
-__device__ __forceinline__ P2 p2_flip(uint2 v, uint32_t f) {
+// (x, y & ymask) with both signs flipped when bit 31 of f is set.
+__device__ __forceinline__ P2 p2_flip(uint2 v, uint32_t f, uint32_t ymask = 0xffffffffu) {
   const uint32_t s = f & 0x80000000u;
   P2 d;
-  asm("mov.b64 %0, {%1, %2};" : "=l"(d) : "r"(v.x ^ s), "r"(v.y ^ s));
+  asm("mov.b64 %0, {%1, %2};" : "=l"(d) : "r"(v.x ^ s), "r"((v.y & ymask) ^ s));
   return d;
 }
 
@@ -113,51 +122,49 @@ struct SrhtArgs {
   float scale;          // 1 for partial sums
 };
 
-// The thread's 32 rows t + 32k of unit rows rbase …, columns c and c + 1.
+// The thread's 32 rows t + 32k of unit rows rbase …, columns c and c + 1.  Lanes
+// past the last column read the first one: nothing of theirs is stored.  With odd
+// d the last column's pair is read whole (8-byte aligned, so it lies in the page
+// of its first half) and the half past the row masked by the caller: a load of
+// its own for that lane made every block of the last slice, and with it the
+// kernel, a sixth slower.
 __device__ __forceinline__ void load_rows(const SrhtArgs& a, long long rbase, int t, int c, uint2 (&v)[32]) {
-  if (rbase + kB <= a.n && (c + 1 < a.d || (c >= a.d && a.d > 1))) {
-    // (lanes past the last column read the first one; nothing of theirs is stored)
-    const char* src = reinterpret_cast<const char*>(a.A + (rbase + t) * a.lda + (c < a.d ? c : 0));
-    long long step = 32 * (long long)sizeof(float) * a.lda;
-    asm volatile("" : "+l"(step));  // (32 precomputed row offsets would take 64 registers)
+  const int col = c < a.d ? c : 0;
+  long long step = 32 * (long long)sizeof(float) * a.lda;
+  asm volatile("" : "+l"(step));  // (32 precomputed row offsets would take 64 registers)
+  if (rbase + kB <= a.n) {
+    const char* src = reinterpret_cast<const char*>(a.A + (rbase + t) * a.lda + col);
 #pragma unroll
     for (int k = 0; k < 32; ++k) {
       v[k] = __ldg(reinterpret_cast<const uint2*>(src));
       src += step;
     }
   } else {
-    // The last rows, or an odd last column, of A.  Eight loads at a time, from
-    // clamped rows and without branches between them (a load behind its own
-    // branch each made the blocks of a ragged last slice run four times as
-    // long as the others).
-    const bool pair = c + 1 < a.d;
-    const char* src =
-        reinterpret_cast<const char*>(a.A + min(rbase + t, (long long)a.n - 1) * a.lda + (c < a.d ? c : 0));
-    long long step = 32 * (long long)sizeof(float) * a.lda;
-    asm volatile("" : "+l"(step));
+    // The last rows of A: eight loads at a time, from clamped rows and without
+    // branches between them.
+    const char* src = reinterpret_cast<const char*>(a.A + min(rbase + t, (long long)a.n - 1) * a.lda + col);
 #pragma unroll
     for (int k8 = 0; k8 < 32; k8 += 8) {
 #pragma unroll
       for (int k = k8; k < k8 + 8; ++k) {
-        if (pair)
-          v[k] = __ldg(reinterpret_cast<const uint2*>(src));
-        else
-          v[k] = make_uint2(__ldg(reinterpret_cast<const unsigned int*>(src)), 0u);
+        v[k] = __ldg(reinterpret_cast<const uint2*>(src));
         if (rbase + t + 32 * (k + 1) < a.n) src += step;
       }
 #pragma unroll
       for (int k = k8; k < k8 + 8; ++k)
-        if (rbase + t + 32 * k >= a.n || c >= a.d) v[k] = make_uint2(0u, 0u);
+        if (rbase + t + 32 * k >= a.n) v[k] = make_uint2(0u, 0u);
       asm volatile("" ::: "memory");
     }
   }
 }
 
-template <int ACC>
+template <int ACC, bool EXTRA>
 __global__ void __launch_bounds__(kThreads, 2) srht_kernel(const SrhtArgs a) {
   extern __shared__ float4 smem4[];
   float* Y = reinterpret_cast<float*>(smem4);                  // kYFloats
   int* off = reinterpret_cast<int*>(Y + kYFloats);             // ACC·32: byte offset of row r_lo in Y
+  int2* xoff = reinterpret_cast<int2*>(off + ACC * 32);        // EXTRA: {offset, r_hi} of the samples past ACC·32
+  P2* xacc = reinterpret_cast<P2*>(xoff + (EXTRA ? a.mc - ACC * 32 : 0));  // … × 8 column pairs: their sums
   const int tid = threadIdx.x, lane = tid & 31;
   const int cl = tid & 7, t = tid >> 3;                        // column pair, row class
   // Slices with the longer ranges come first: two of them never share an SM.
@@ -185,6 +192,14 @@ __global__ void __launch_bounds__(kThreads, 2) srht_kernel(const SrhtArgs a) {
     const int i = i0 + e;
     off[e] = i < i1 ? 4 * y_off(a.rows[i] & (kB - 1)) : 0;
   }
+  const int nx = EXTRA ? max(0, i1 - i0 - ACC * 32) : 0;
+  if (EXTRA) {
+    for (int e = tid; e < nx; e += kThreads) {
+      const int r = a.rows[i0 + ACC * 32 + e];
+      xoff[e] = make_int2(4 * y_off(r & (kB - 1)), r >> kLB);
+    }
+    for (int e = t; e < nx; e += 32) xacc[8 * e + cl] = 0ull;  // (read and added to by this thread only)
+  }
   constexpr int NJ = (ACC + 7) / 8;
   int rhi[NJ];
 #pragma unroll
@@ -197,6 +212,7 @@ __global__ void __launch_bounds__(kThreads, 2) srht_kernel(const SrhtArgs a) {
   for (int q = 0; q < ACC; ++q) acc[q] = 0ull;
   const char* Yc = reinterpret_cast<const char*>(Y) + 8 * cl;
   const int nwords = (a.n + 31) >> 5;
+  const uint32_t ymask = c + 1 < a.d ? 0xffffffffu : 0u;
 
   uint2 v[32];
   for (int blk = b0 - 1; blk < b1; ++blk) {
@@ -213,7 +229,7 @@ __global__ void __launch_bounds__(kThreads, 2) srht_kernel(const SrhtArgs a) {
       if ((t & 3) == r) neg = bal;
     }
 #pragma unroll
-    for (int k = 0; k < 32; ++k) x[k] = p2_flip(v[k], neg << (31 - k));
+    for (int k = 0; k < 32; ++k) x[k] = p2_flip(v[k], neg << (31 - k), ymask);
     fwht32(x);  // the high five bits of the row
     __syncthreads();  // the previous unit's sampled rows have been read
     P2* Yt = reinterpret_cast<P2*>(Y + y_off(t) + 2 * cl);
@@ -248,6 +264,14 @@ __global__ void __launch_bounds__(kThreads, 2) srht_kernel(const SrhtArgs a) {
       const uint2 y = *reinterpret_cast<const uint2*>(Yc + off[q * 32 + t]);
       acc[q] = p2_add(acc[q], p2_flip(y, sg[q >> 3] << (31 - (q & 7))));
     }
+    if (EXTRA) {
+#pragma unroll 4
+      for (int e = t; e < nx; e += 32) {
+        const int2 o = xoff[e];
+        const uint2 y = *reinterpret_cast<const uint2*>(Yc + o.x);
+        xacc[8 * e + cl] = p2_add(xacc[8 * e + cl], p2_flip(y, (uint32_t)__popc(o.y & blk) << 31));
+      }
+    }
   }
   float* out = a.out + (long long)range * a.m * a.ldo;
 #pragma unroll
@@ -257,6 +281,14 @@ __global__ void __launch_bounds__(kThreads, 2) srht_kernel(const SrhtArgs a) {
     asm("mov.b64 {%0, %1}, %2;" : "=f"(v2.x), "=f"(v2.y) : "l"(acc[q]));
     if (i < i1) {
       float* o = out + (long long)i * a.ldo + c;
+      if (c < a.d) o[0] = v2.x * a.scale;
+      if (c + 1 < a.d) o[1] = v2.y * a.scale;
+    }
+  }
+  if (EXTRA) {
+    for (int e = t; e < nx; e += 32) {
+      const float2 v2 = *reinterpret_cast<const float2*>(xacc + 8 * e + cl);
+      float* o = out + (long long)(i0 + ACC * 32 + e) * a.ldo + c;
       if (c < a.d) o[0] = v2.x * a.scale;
       if (c + 1 < a.d) o[1] = v2.y * a.scale;
     }
@@ -279,11 +311,12 @@ __global__ void __launch_bounds__(256) srht_reduce_kernel(const float* __restric
 using KernelFn = void (*)(const SrhtArgs);
 
 KernelFn pick_kernel(int acc) {
-  if (acc <= 4) return srht_kernel<4>;
-  if (acc <= 8) return srht_kernel<8>;
-  if (acc <= 12) return srht_kernel<12>;
-  if (acc <= 16) return srht_kernel<16>;
-  return srht_kernel<kAccMax>;
+  if (acc <= 4) return srht_kernel<4, false>;
+  if (acc <= 8) return srht_kernel<8, false>;
+  if (acc <= 12) return srht_kernel<12, false>;
+  if (acc <= 16) return srht_kernel<16, false>;
+  if (acc <= kAccMax) return srht_kernel<kAccMax, false>;
+  return srht_kernel<kAccMax, true>;
 }
 int acc_slots(int acc) { return acc <= 16 ? (acc + 3) / 4 * 4 : kAccMax; }
 
@@ -300,7 +333,8 @@ int sketch_srht(const float* A, int64_t n, int64_t d, int64_t lda, int64_t m, ui
   const int nblk = (int)((n + kB - 1) / kB);
   const int ncs = (int)((d + kW - 1) / kW);
   // Samples per block: as many as the registers hold, evenly cut.
-  const int zc = (int)((m + kAccMax * 32 - 1) / (kAccMax * 32));
+  const int per_block = kAccMax * 32 + kExtra;
+  const int zc = (int)((m + per_block - 1) / per_block);
   const int mc = (int)round_up((m + zc - 1) / zc, 32);
   // The blocks of one column slice share its units.  All slices are walked in
   // step (neighbours read the two halves of a 128-byte line within a short
@@ -347,7 +381,9 @@ int sketch_srht(const float* A, int64_t n, int64_t d, int64_t lda, int64_t m, ui
   a.scale = ranges > 1 ? 1.f : scale;
   const int acc = mc / 32;
   const KernelFn fn = pick_kernel(acc);
-  const size_t smem = sizeof(float) * kYFloats + sizeof(int) * 32 * (size_t)acc_slots(acc);
+  const size_t extra = acc > kAccMax ? (size_t)(mc - kAccMax * 32) : 0;
+  const size_t smem = sizeof(float) * kYFloats + sizeof(int) * 32 * (size_t)acc_slots(acc) +
+                      (sizeof(int2) + sizeof(float) * kW) * extra;
   MIHS_CUDA_TRY(cudaFuncSetAttribute((const void*)fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
   fn<<<(unsigned)((ncs * ks + wide) * zc), kThreads, smem, s>>>(a);
   MIHS_CHECK_LAUNCH();

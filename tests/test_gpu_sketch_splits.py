@@ -48,3 +48,12 @@ def test_srht_splits_are_exact(n, d, m):
     ref = o.sketch_apply(o.SRHT, A[:, :d].numpy().astype(np.float64), m, 5 + m)
     sums = np.rint(ref * np.sqrt(m))  # the integers themselves (the oracle's own fp64 rounding dropped)
     assert np.all(np.abs(SA * np.sqrt(m) - sums) <= 2.0 ** -22 * np.abs(sums))
+
+
+# n, d, m: the samples that a block holds in registers and one more (their sums then lie in shared memory), as many of
+# both as one block takes and the first that take two, with an odd last column and with that column alone, units that
+# end inside the matrix and that do not
+@pytest.mark.parametrize("n,d,m", [(5000, 33, 640), (5000, 33, 641), (4096, 17, 673), (3000, 1, 700), (5000, 15, 1240),
+                                   (6000, 16, 1241), (4100, 1023, 1249), (9001, 31, 1300), (20000, 2, 2481)])
+def test_srht_samples_past_the_registers(n, d, m):
+    test_srht_splits_are_exact(n, d, m)
