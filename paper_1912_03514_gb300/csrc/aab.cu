@@ -19,8 +19,8 @@
 // The d-vectors of the recursion (v, d, x) are replicated per block (O(d)
 // work, negligible next to the O(md/CL) products).
 //
-// That is the form for sketches whose rows fit the shared memory of a cluster
-// but not its registers; aab_reg.cuh, which is faster (68 against 141 µs for 30
+// That is the form for sketches that fit the shared memory of a cluster but
+// not its registers; aab_reg.cuh, which is faster (68 against 141 µs for 30
 // passes at 588 × 1024), takes all that do.  When SA is too large for
 // the shared memory of 16 blocks, launch_aab hands a single-λ solve that has
 // scratch to the grid form (aab_grid.cu); otherwise the cluster's blocks
@@ -84,7 +84,7 @@ int smem_pitch(int dp, int sa_type) { return sa_type == MIHS_SA_FP32 ? dp : (int
 size_t smem_bytes(int m, int dp, int cl, bool in_smem, int sa_type) {
   const int rpc = (m + cl - 1) / cl;
   const int rpc_pad = (int)round_up(rpc, 4);
-  size_t base = (size_t)((5 + kWarps) * dp + 2 * rpc_pad + kWarps + 8) * sizeof(float);
+  size_t base = ((size_t)(5 * dp + 2 * rpc_pad + kWarps + 8) + wpart_floats(dp)) * sizeof(float);
   if (in_smem) base += (size_t)rpc * smem_pitch(dp, sa_type) * elem_bytes(sa_type);
   return base;
 }

@@ -173,6 +173,17 @@ def test_grid_solves_reach_the_solution(grid_form, family):
     assert mihs.device_status() == 0
 
 
+@pytest.mark.parametrize("m,d", [(100000, 3), (90000, 4)])
+def test_cluster_of_a_tall_and_narrow_sketch(m, d):
+    """16 blocks with SA in shared memory and slices of four columns: their 16 shares of a slice outnumber the eight
+    warps' sums of all columns, whose place they take."""
+    SA, g = _sa_case(m, d, 77)
+    amp, ref = _amp(SA.numpy().astype(np.float64), g.numpy().astype(np.float64), 0.3, d)
+    delta = mihs.aab_solve(SA.to(DEV), g.to(DEV), 0.3, eps_sub=0.0)
+    assert o.rel_error(_np(delta), ref) <= 20 * max(amp, 4 * U32 * math.sqrt(m))
+    assert mihs.device_status() == 0
+
+
 # ---------------- one cluster reading SA from global memory (L2)
 @pytest.mark.parametrize("m,d,lam,k", [(4096, 1024, 1e-3, 12), (3000, 700, 1e-2, 25), (5000, 512, 0.05, 7)])
 def test_cluster_global_sa_matches_oracle(monkeypatch, m, d, lam, k):
