@@ -156,9 +156,12 @@ __global__ void __launch_bounds__(kThreads, 1) aab_gridreg_kernel(const GridRegP
   __shared__ float scal;                 // ρ²
   SolveCtl* ctl = P.ctl;
 
-  // The control block is written by block 0 only, once every block has read it: at
-  // the end (it has then finished a pass, with shares from every block), or, where
-  // the launch makes no pass, after all_have_read().
+  // The control block is written by block 0 only: at the end (every block has
+  // then read it, or block 0 could not have finished a pass), or when the solve
+  // stops, while others may still be reading it.  Those that see `done` leave; to
+  // the others the values written are the ones that they have or compute: until
+  // ‖g(0)‖ is known gnorm0 is negative, so that gnorm0_known read without the
+  // gnorm0 that belongs to it counts for nothing.
   int done = 0, outer = 0, max_outer = 0, g0known = 0, phase = 1, refresh = 1, corr = 0;
   float tol = 0.f, gnorm0 = 0.f, switch_tol = 0.f;
   if (ctl != nullptr) {
@@ -173,7 +176,7 @@ __global__ void __launch_bounds__(kThreads, 1) aab_gridreg_kernel(const GridRegP
     refresh = ctl->refresh;
     corr = ctl->corr;
   }
-  done = __syncthreads_or(done);  // (one decision per block, should another's wait have run out already)
+  done = __syncthreads_or(done);  // (one decision per block)
   if (done) {
     if (P.cond != 0ull && blk == 0 && tid == 0) cudaGraphSetConditional((cudaGraphConditionalHandle)P.cond, 0u);
     return;
@@ -225,36 +228,8 @@ __global__ void __launch_bounds__(kThreads, 1) aab_gridreg_kernel(const GridRegP
   float zo = own && jo < d ? P.g[jo] : 0.f, dv = 0.f, xs = 0.f;
   const float theta1 = sqrtf(block_sum(gsq, bsum));
 
-  // Every block gets here after its threads have read the control block (the
-  // block sum above): it says so with a ρ² word, and block 0 waits for all of
-  // them.  False in block 0 when that wait ran out.
-  auto all_have_read = [&]() {
-    bool all = true;
-    if (tid == 0) st_word(P.rho + blk, word(0.f, base + 1u));
-    if (blk == 0) {
-      Poll poll;
-      for (int b = tid; b < G && all; b += kThreads)
-        while (!ready(ld_word(P.rho + b), base + 1u))
-          if (!poll.again()) {
-            all = false;
-            break;
-          }
-    }
-    return !__syncthreads_or(!all);
-  };
-  auto time_out = [&]() {
-    if (tid == 0) {
-      atomicExch(&g_aab_gridreg_error, MIHS_ERR_TIMEOUT);
-      if (ctl != nullptr) {
-        ctl->status = MIHS_ERR_TIMEOUT;
-        ctl->done = 1;
-      }
-      if (P.cond != 0ull) cudaGraphSetConditional((cudaGraphConditionalHandle)P.cond, 0u);
-    }
-  };
-
   if (ctl != nullptr) {  // stop test of Algorithm 1 on ‖g‖ = θ₁
-    const float g0 = g0known ? gnorm0 : theta1;
+    const float g0 = g0known && gnorm0 >= 0.f ? gnorm0 : theta1;
     if (P.hist != nullptr && blk == 0 && tid == 0 && outer < kHistCap) P.hist[outer] = theta1;
     const bool bad = !(theta1 <= 3.0e38f);
     // A refinement correction's gradient is approximate: it never stops the
@@ -264,11 +239,7 @@ __global__ void __launch_bounds__(kThreads, 1) aab_gridreg_kernel(const GridRegP
     const bool correction = phase == 1 && corr && !refresh;
     const bool conv = tol > 0.f && theta1 <= tol * g0 && !correction && phase != 0;
     const bool capped = outer >= max_outer;
-    if (bad || conv || capped) {  // the same in every block
-      if (!all_have_read()) {
-        time_out();
-        return;
-      }
+    if (bad || conv || capped) {
       if (blk == 0 && tid == 0) {
         ctl->gnorm = theta1;
         ctl->gnorm0 = g0;
@@ -518,11 +489,32 @@ __global__ void __launch_bounds__(kThreads, 1) aab_gridreg_kernel(const GridRegP
       if (!(t >= P.eps && k < P.max_passes && rho > 0.f)) break;  // the same in every block
     }
   }
-  if (!(theta1 > 0.f)) failed = !all_have_read();  // nothing to do
+  if (!(theta1 > 0.f)) {
+    // Nothing to do, but block 0 may write the control block only once every
+    // block has read it.
+    if (tid == 0) st_word(P.rho + blk, word(0.f, base + 1u));
+    if (blk == 0) {
+      Poll poll;
+      for (int b = tid; b < G && ok; b += kThreads)
+        while (!ready(ld_word(P.rho + b), base + 1u))
+          if (!poll.again()) {
+            ok = false;
+            break;
+          }
+    }
+    failed = __syncthreads_or(!ok) != 0;
+  }
   // (all that write it write the same; it wraps at 2³²)
   if (tid == 0 && (failed || blk == 0)) atomicExch(P.epoch, base + kEpochStep);
   if (failed) {
-    time_out();
+    if (tid == 0) {
+      atomicExch(&g_aab_gridreg_error, MIHS_ERR_TIMEOUT);
+      if (ctl != nullptr) {
+        ctl->status = MIHS_ERR_TIMEOUT;
+        ctl->done = 1;
+      }
+      if (P.cond != 0ull) cudaGraphSetConditional((cudaGraphConditionalHandle)P.cond, 0u);
+    }
     return;
   }
 

@@ -88,6 +88,7 @@ __global__ void ctl_init_kernel(SolveCtl* ctl, int max_outer, float tol, int pha
   c.max_outer = max_outer;
   c.tol = tol;
   c.status = MIHS_OK;
+  c.gnorm0 = -1.f;
   c.phase = phase;
   c.switch_tol = switch_tol;
   c.gmin = 3.0e38f;

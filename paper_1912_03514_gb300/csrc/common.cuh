@@ -63,7 +63,7 @@ struct SolveCtl {
   int max_outer;
   int gnorm0_known;  // ‖Aᵀb‖ already in gnorm0
   float tol;         // stop when ‖g‖ ≤ tol·‖Aᵀb‖
-  float gnorm0;      // ‖Aᵀb‖
+  float gnorm0;      // ‖Aᵀb‖; negative until known (single-λ solves)
   float gnorm;       // ‖g‖ of the current x
   int phase;         // refinement solves: 0 = plain fp32 gradient, 1 = compensated
   float switch_tol;  // switch to phase 1 once ‖g‖ ≤ switch_tol·‖Aᵀb‖ ...

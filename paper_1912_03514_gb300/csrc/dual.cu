@@ -249,6 +249,7 @@ __global__ void dual_ctl_init_kernel(SolveCtl* ctl, int max_outer, float tol) {
   SolveCtl c = {};
   c.max_outer = max_outer;
   c.tol = tol;
+  c.gnorm0 = -1.f;
   c.status = MIHS_OK;
   c.phase = 1;
   c.gmin = 3.0e38f;
