@@ -552,6 +552,13 @@ __global__ void __launch_bounds__(kThreads, 1) aab_gridreg_kernel(const GridRegP
 
 using GridRegFn = void (*)(const GridRegParams);
 
+// Rows of SA held, the smallest that fits: a pass costs what is held, not what
+// is used.  At one group of columns up to 28 rows, the most that the 32 lanes of
+// the dots and groups of four rows leave room for (30 passes, 1000 columns: 120 µs
+// with 3040 rows, 20 a block, 129 with 3041 in the kernel of 28).  At two, 24 rows
+// spill 0.5 KB a thread and 21 0.2 KB: 2048 columns take 141 µs with 2433 to 3192
+// rows (17 to 21 a block), 178 with 3193; in the shared-memory form 220, 228 and
+// 232, and 983 with 3600 rows, which are past its shared memory.
 GridRegFn gridreg_kernel(int dp, int rows) {
   if (dp > 1024) {
     if (rows <= 8) return aab_gridreg_kernel<2, 8>;

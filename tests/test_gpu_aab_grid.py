@@ -134,6 +134,29 @@ def test_grid_aab_quantised_sa(grid_form, m, d, lam, prec):
     assert err <= 20 * max(amp, 4 * U32 * math.sqrt(d)), (err, amp)
 
 
+# rows per block on both sides of every step of the register form, at both of its widths, and past it, where each
+# storage type is held in shared memory (8 blocks, the last one short of rows)
+ROW_STEPS = [(r, d) for d in (700, 2045) for r in (7, 8, 9, 16, 17, 20, 21, 22, 24, 25, 28, 29)] + [(33, 1024)]
+
+
+@pytest.mark.parametrize("prec", ["fp32", "bf16", "fp8"])
+@pytest.mark.parametrize("rows,d", ROW_STEPS)
+def test_grid_aab_rows_per_block(grid_form, monkeypatch, rows, d, prec):
+    monkeypatch.setenv("MIHS_AAB_GRID_BLOCKS", "8")
+    m, lam, k = 8 * rows - 3, 0.1, 5
+    SA, g = _sa_case(m, d, 13 * m + d)
+    if prec == "fp32":
+        SAd = SA.numpy().astype(np.float64)
+        delta = mihs.aab_solve(SA.to(DEV), g.to(DEV), lam, eps_sub=0.0, max_inner=k)
+    else:
+        q, sc = mihs.quantize_sa(SA.to(DEV), prec)
+        SAd = _decoded(q, sc, prec, m, d)
+        delta = mihs.aab_solve_q(q, prec, sc, d, g.to(DEV), lam, eps_sub=0.0, max_inner=k)
+    amp, ref = _amp(SAd, g.numpy().astype(np.float64), lam, k)
+    assert o.rel_error(_np(delta), ref) <= 20 * max(amp, 4 * U32 * math.sqrt(d))
+    assert mihs.device_status() == 0
+
+
 def test_grid_aab_heavy_ball(grid_form):
     m, d, lam, k = 588, 1024, 1e-3, 6
     sd = 0.3 * min(m, d)
