@@ -137,3 +137,12 @@ def test_gradients_are_exact(n, d):
     ref = An.T @ (b.double().numpy() - An @ x.double().numpy()) - 3.0 * x.double().numpy()
     assert np.array_equal(mihs.gradient(A, b.to(DEV), x.to(DEV), 3.0).cpu().double().numpy(), ref)
     assert np.array_equal(mihs.gradient_refined(A, b.to(DEV), x.double().to(DEV), 3.0).cpu().numpy(), ref)
+
+
+# rows of dA off 16 bytes: the widths at which the last 128 columns are half full and one fewer, for each count of such
+# groups, and past them
+@pytest.mark.parametrize("n,d", [(300, 63), (301, 65), (77, 191), (78, 193), (100, 319), (101, 321), (65, 447), (66, 449),
+                                 (64, 575), (63, 577), (65, 703), (64, 705), (33, 831), (34, 833), (33, 959), (32, 961),
+                                 (40, 1023), (41, 1087), (42, 1089)])
+def test_backward_of_unaligned_rows(n, d):
+    test_backward_is_exact(n, d)
