@@ -177,7 +177,8 @@ __global__ void atnu_reduce_kernel(const float* __restrict__ part, int nsplit, l
 // A_i·u over a column slice for kResidRows rows per block (each load of u
 // serves them all), fixed-order block sums: part[slice][i], or with one slice
 // g_i = b_i − A_i·u − λν_i at once.  Slices only where four rows per block do
-// not make three blocks per SM (128×200000: 32 blocks, both passes 183 µs; cut
+// not make more than two blocks per SM (1216×65536 cut in two: 113 µs, whole 123;
+// 1300×65536: 136 and 126; 128×200000: 32 blocks, both passes 183 µs; cut
 // into slices, with the other pass below its 30 µs of HBM time, 47 µs).
 constexpr int kResidRows = 4;
 
@@ -196,7 +197,6 @@ __global__ void __launch_bounds__(kT) dual_resid_kernel(const float* __restrict_
   const float* rows[kResidRows];
 #pragma unroll
   for (int r = 0; r < kResidRows; ++r) rows[r] = A + (long long)min(i0 + r, n - 1) * lda;
-#pragma unroll 2
   for (int k = k0 + threadIdx.x; k < k1; k += kT) {
     const float4 v = __ldcg(reinterpret_cast<const float4*>(u) + k);
 #pragma unroll
@@ -281,9 +281,14 @@ DualPlan dual_plan(int64_t n, int64_t d) {
   p.rows = (int)round_up((n + splits - 1) / splits, kAtnuStageRows);
   if (p.rows > kAtnuRows) p.rows = kAtnuRows;
   p.splits = (int)((n + p.rows - 1) / p.rows);
+  if (n <= kAtnuRows && n * d <= (2 << 20)) {  // a few MB: bound by launches, so one less
+    p.rows = (int)round_up(n, kAtnuStageRows);
+    p.splits = 1;
+  }
   const int64_t quads = (n + kResidRows - 1) / kResidRows;
-  int64_t slices = quads >= 3LL * num_sms() ? 1 : (4LL * num_sms() + quads - 1) / quads;
+  int64_t slices = quads > 2LL * num_sms() ? 1 : (4LL * num_sms() + quads - 1) / quads;
   if (slices > d / 4096) slices = d / 4096;                 // at least 16 KB of a row each
+  if (n * d <= (4 << 20)) slices = 1;                       // (one launch less again)
   if (slices < 1) slices = 1;
   p.cols = (int)round_up((d + slices - 1) / slices, 4);
   p.slices = (int)((d + p.cols - 1) / p.cols);
@@ -297,19 +302,21 @@ size_t dual_scratch_floats(int64_t n, int64_t d) {
   return (size_t)p.splits * (size_t)round_up(d, 4) + (size_t)p.slices * (size_t)round_up(n, 4);
 }
 
-// u = Aᵀν through row-split partials in `scratch`.
+// u = Aᵀν through row-split partials in `scratch` (u itself where one split has all rows).
 int launch_atnu(const float* A, int64_t n, int64_t d, int64_t lda, const float* nu, float* u, float* scratch,
                 SolveCtl* ctl, cudaStream_t s) {
   const DualPlan p = dual_plan(n, d);
   const long long ldp = round_up(d, 4);
   const unsigned cblocks = (unsigned)((d + kAtnuCols - 1) / kAtnuCols);
   MIHS_CUDA_TRY(cudaFuncSetAttribute(atnu_partial_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kAtnuSmem));
-  atnu_partial_kernel<<<dim3(cblocks, (unsigned)p.splits), kT + 32, kAtnuSmem, s>>>(A, (int)n, (int)d, lda, nu, scratch,
-                                                                                    ldp, p.rows, ctl);
+  atnu_partial_kernel<<<dim3(cblocks, (unsigned)p.splits), kT + 32, kAtnuSmem, s>>>(
+      A, (int)n, (int)d, lda, nu, p.splits == 1 ? u : scratch, ldp, p.rows, ctl);
   MIHS_CHECK_LAUNCH();
+  count_launch();
+  if (p.splits == 1) return MIHS_OK;
   atnu_reduce_kernel<<<(unsigned)((d + 255) / 256), 256, 0, s>>>(scratch, p.splits, ldp, (int)d, u, ctl);
   MIHS_CHECK_LAUNCH();
-  count_launch(2);
+  count_launch();
   return MIHS_OK;
 }
 

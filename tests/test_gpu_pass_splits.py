@@ -146,3 +146,10 @@ def test_gradients_are_exact(n, d):
                                  (40, 1023), (41, 1087), (42, 1089)])
 def test_backward_of_unaligned_rows(n, d):
     test_backward_is_exact(n, d)
+
+
+# n, d: one split that writes A^T nu itself, the first matrix with two, one column slice and more
+@pytest.mark.parametrize("n,d", [(256, 1500), (257, 1500), (128, 16384), (129, 16384), (255, 8193), (300, 16381),
+                                 (64, 65536), (64, 65540)])
+def test_dual_gradient_of_few_rows(n, d):
+    test_dual_gradient_is_exact(n, d)
