@@ -34,7 +34,9 @@
 // barriers per 16 rows for, whatever nl.  Whole call, before → after, with 16 / 8 /
 // 4 iterates: 65536×512 101 → 91 / 61 / 57 µs, 65536×1024 153 → 151 / 100 / –,
 // 60000×700 140 → 134 / 83 / 67, 200000×129 141 → 127 / 81 / 68, 100000×256
-// 96 → 76 / 51 / 45, 262144×64 114 → 100 / 66 / 49.
+// 96 → 76 / 51 / 45, 262144×64 114 → 100 / 66 / 49.  Column warps cover 256 columns
+// and iterates go by 8, so just past such a step half of both is padding: there,
+// with more than 8 iterates, the form of apass_path_smem.cu is the faster one.
 //
 // Per-block column sums go to partials[block][l][j]; a finalize kernel adds
 // them in a fixed order and subtracts λ_l·X[l].
@@ -353,28 +355,41 @@ apass_path_kernel(const float* __restrict__ A, int n, int d, long long lda, cons
   }
 }
 
-// G[l][j] = Σ_p partials[p][l][j] − λ_l·X[l][j] (fixed order), l < nl.
-__global__ void apass_path_finalize_kernel(const float* __restrict__ partials, int P, int d, int dpad,
-                                           const float* __restrict__ X, long long ldx, PathScalars sc,
-                                           float* __restrict__ G, long long ldg, const int* __restrict__ all_done) {
+// G[l][j] = Σ_p partials[p][l][j] − λ_l·X[l][j] (fixed order), l < nl.  A block
+// adds C columns in 256/C groups of partials.
+template <int C>
+__global__ void __launch_bounds__(256)
+apass_path_finalize_kernel(const float* __restrict__ partials, int P, int d, int dpad, const float* __restrict__ X,
+                           long long ldx, PathScalars sc, float* __restrict__ G, long long ldg,
+                           const int* __restrict__ all_done) {
   if (all_done != nullptr && *all_done) return;
   const int l = blockIdx.y;
   if (l >= sc.nl) return;
-  __shared__ float red[32][9];  // 8 columns × 32 partial groups per block
-  const int c = threadIdx.x & 7, grp = threadIdx.x >> 3;
-  const int col = blockIdx.x * 8 + c;
+  constexpr int NG = 256 / C;
+  __shared__ float red[NG][C + 1];
+  const int c = threadIdx.x % C, grp = threadIdx.x / C;
+  const int col = blockIdx.x * C + c;
   float s = 0.f;
   if (col < d) {
 #pragma unroll 8
-    for (int p = grp; p < P; p += 32) s += partials[((size_t)p * kL + l) * dpad + col];
+    for (int p = grp; p < P; p += NG) s += partials[((size_t)p * kL + l) * dpad + col];
   }
   red[grp][c] = s;
   __syncthreads();
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  const int j = blockIdx.x * 8 + warp;
-  const float t = warp_sum(red[lane][warp]);
-  if (lane == 0 && j < d)
-    G[(long long)l * ldg + j] = t - (X != nullptr ? sc.lam[l] * X[(long long)l * ldx + j] : 0.f);
+  float t = 0.f;
+  int j;
+  if constexpr (C == 8) {  // one warp per column
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    j = lane == 0 ? blockIdx.x * C + warp : d;
+    t = warp_sum(red[lane][warp]);
+  } else {
+    j = grp == 0 ? col : d;
+    if (grp == 0) {
+#pragma unroll
+      for (int k = 0; k < NG; ++k) t += red[k][c];
+    }
+  }
+  if (j < d) G[(long long)l * ldg + j] = t - (X != nullptr ? sc.lam[l] * X[(long long)l * ldx + j] : 0.f);
 }
 
 }  // namespace
@@ -404,6 +419,15 @@ PathKernel path_kernel_for(int64_t dpad) {
   return {(const void*)&apass_path_kernel<KI, 4, 2>, 4, path_max_warps(KI, 2)};
 }
 
+// More than eight iterates at widths just past one of the register form's steps
+// (both sides of the lines stand in apass_path_smem.cu), and rows enough for the
+// block's start, which fills X's 16 rows of shared memory.
+bool path_in_smem(int64_t n, int64_t dpad, int nl) {
+  if (nl <= 8) return false;
+  if (dpad > 256 && dpad <= 384) return n >= 12288;
+  return dpad > 512 && (dpad <= 640 || (dpad <= 832 && n >= 32768));
+}
+
 }  // namespace
 
 int launch_apass_path(const float* A, int64_t n, int64_t d, int64_t lda, const float* b, const float* X,
@@ -413,6 +437,7 @@ int launch_apass_path(const float* A, int64_t n, int64_t d, int64_t lda, const f
     set_error("path A-pass: d=%lld (max %d) or nl=%d (1..%d) unsupported", (long long)d, kPathMaxD, nl, kL);
     return MIHS_ERR_UNSUPPORTED;
   }
+  if (path_in_smem(n, dpad, nl)) return launch_apass_path_smem(A, n, d, lda, b, X, ldx, nl, partials, all_done, s);
   const int P = apass_path_num_partials(n);
   const int rows_per_cta = (int)round_up((n + P - 1) / P, kStageRows);
   const int its = nl <= 4 ? 4 : 8;
@@ -437,8 +462,11 @@ int launch_apass_path(const float* A, int64_t n, int64_t d, int64_t lda, const f
 int launch_apass_path_finalize(const float* partials, int P, int64_t d, const float* X, int64_t ldx,
                                const PathScalars& sc, float* G, int64_t ldg, const int* all_done,
                                cudaStream_t s) {
-  apass_path_finalize_kernel<<<dim3((unsigned)((d + 7) / 8), (unsigned)sc.nl), 256, 0, s>>>(
-      partials, P, (int)d, (int)apass_dpad(d), X, ldx, sc, G, ldg, all_done);
+  // 32 columns read whole sectors; 8 spread few sums over more SMs
+  const int c = (d + 31) / 32 * sc.nl >= num_sms() ? 32 : 8;
+  auto kern = c == 32 ? apass_path_finalize_kernel<32> : apass_path_finalize_kernel<8>;
+  kern<<<dim3((unsigned)((d + c - 1) / c), (unsigned)sc.nl), 256, 0, s>>>(partials, P, (int)d, (int)apass_dpad(d), X,
+                                                                          ldx, sc, G, ldg, all_done);
   MIHS_CHECK_LAUNCH();
   count_launch();
   return MIHS_OK;
@@ -448,7 +476,10 @@ int apass_path_device_error(int* code) {
   int v = 0, z = 0;
   MIHS_CUDA_TRY(cudaMemcpyFromSymbol(&v, g_apass_path_error, sizeof(int)));
   MIHS_CUDA_TRY(cudaMemcpyToSymbol(g_apass_path_error, &z, sizeof(int)));
-  *code = v;
+  int w = 0;
+  const int rc = apass_path_smem_device_error(&w);
+  if (rc) return rc;
+  *code = v ? v : w;
   return MIHS_OK;
 }
 

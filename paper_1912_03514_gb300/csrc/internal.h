@@ -48,6 +48,11 @@ int apass_path_max_d();
 // all work when *all_done (may be NULL).
 int launch_apass_path(const float* A, int64_t n, int64_t d, int64_t lda, const float* b, const float* X,
                       int64_t ldx, int nl, float* partials, const int* all_done, cudaStream_t s);
+// The same in its shared-memory form (apass_path_smem.cu), which launch_apass_path
+// chooses by nl and d.
+int launch_apass_path_smem(const float* A, int64_t n, int64_t d, int64_t lda, const float* b, const float* X,
+                           int64_t ldx, int nl, float* partials, const int* all_done, cudaStream_t s);
+int apass_path_smem_device_error(int* code);
 // G[l][j] = Σ_p partials[p][l][j] − λ_l·X[l][j] (fixed order), G λ-major (ldg).
 int launch_apass_path_finalize(const float* partials, int P, int64_t d, const float* X, int64_t ldx,
                                const PathScalars& sc, float* G, int64_t ldg, const int* all_done,

@@ -153,3 +153,13 @@ def test_backward_of_unaligned_rows(n, d):
                                  (64, 65536), (64, 65540)])
 def test_dual_gradient_of_few_rows(n, d):
     test_dual_gradient_is_exact(n, d)
+
+
+# more than eight iterates on both sides of each width, and each number of rows, at which the pass keeps them in shared
+# memory
+@pytest.mark.parametrize("n,d,nl", [(13000, 256, 9), (12289, 257, 9), (12288, 300, 16), (12287, 300, 16), (14001, 381, 10),
+                                    (14000, 384, 9), (13000, 385, 9), (2001, 512, 12), (2500, 513, 9), (2499, 600, 16),
+                                    (37, 640, 11), (3, 540, 13), (2000, 641, 9), (32768, 645, 9), (32767, 700, 16),
+                                    (33001, 701, 12), (32769, 832, 9), (33000, 833, 9)])
+def test_path_gradient_of_many_iterates(n, d, nl):
+    test_path_gradient_is_exact(n, d, nl)
