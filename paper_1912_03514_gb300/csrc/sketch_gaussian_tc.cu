@@ -47,8 +47,9 @@ constexpr int TM = 128;          // sketch rows per tile (MMA M)
 constexpr int TN = 256;          // columns of A per tile (MMA N)
 constexpr int TK = 32;           // rows of A per TMA load (a tf32 stage: 4 MMAs of K = 8)
 constexpr int kGenWarps = 16;    // S generators (warps 2–17); warps 2–5 then run the epilogue
-constexpr int kTrWarps = 8;      // A transposers (warps 18–25), one column of the tile per thread
-constexpr int kThreads = (2 + kGenWarps + kTrWarps) * 32;  // warp 0: MMA, warp 1: TMA
+// A transposers (warps 18 …), two columns of the tile per thread, or one (EARLY)
+constexpr int tr_warps(bool early) { return early ? 8 : 4; }
+constexpr int tc_threads(bool early) { return (2 + kGenWarps + tr_warps(early)) * 32; }  // warp 0: MMA, warp 1: TMA
 constexpr uint32_t kSBytes = TM * TK * 4;       // one 128-row S tile: 16 KB
 constexpr uint32_t kABytes = TK * TN * 4;       // one 32-row fp32 A tile: 32 KB
 
@@ -234,8 +235,14 @@ struct GaussTcArgs {
 // bf16 (kind::f16, 64 K per stage, two TMA loads of 32 rows); 2: S and the
 // scaled A rounded to e4m3 (kind::f8f6f4, 128 K per stage, four loads).
 // MT sketch-row tiles of 128 per block, one TMEM accumulator each.
-template <int PREC, int MT>
-__global__ void __launch_bounds__(kThreads, 1)
+//
+// EARLY: the generators and the transposers make a stage's operands ready in
+// registers before they wait for the stage, so that only the stores lie between
+// the last MMA on it and the next; twice the transposers, one column each.  That
+// shortens the handoff at the price of more instructions; which of the two
+// bounds a cluster depends on its shape (early_operands).
+template <int PREC, int MT, bool EARLY>
+__global__ void __launch_bounds__(tc_threads(EARLY), 1)
 gauss_tc_kernel(const __grid_constant__ CUtensorMap tmap_a, const GaussTcArgs a) {
   using C = TcCfg<PREC, MT>;
   constexpr int KT = C::KT;
@@ -244,6 +251,7 @@ gauss_tc_kernel(const __grid_constant__ CUtensorMap tmap_a, const GaussTcArgs a)
   constexpr int NSTG = C::NSTG;
   constexpr uint32_t kStageBytes = C::StageBytes;
   constexpr int MROWS = MT * TM;   // sketch rows of the block
+  constexpr int kTrWarps = tr_warps(EARLY);
   extern __shared__ unsigned char smem_raw[];
   // 1024-byte alignment for the 128-byte swizzle atoms.
   unsigned char* base = reinterpret_cast<unsigned char*>(
@@ -356,15 +364,46 @@ gauss_tc_kernel(const __grid_constant__ CUtensorMap tmap_a, const GaussTcArgs a)
     __syncwarp();
   } else if (warp >= 2 + kGenWarps) {
     // ------------------------------------------------ A transposers: staging → K-major
-    // The stage's column is loaded and rounded before the wait for the stage: only
-    // the stores are left when its last MMAs have read it.  With the same order in
-    // the generators, S·A of 262144×1024 to 1024 rows went from 962 to 925 µs.
-    const int c = threadIdx.x - (2 + kGenWarps) * 32;  // column 0..255
+    constexpr int NCOL = TN / (kTrWarps * 32);        // columns per thread, kTrWarps·32 apart
+    const int tt = threadIdx.x - (2 + kGenWarps) * 32;
     const float as = PREC == 2 ? a.ascale[0] : 1.f;
+    // 16-byte chunks ch0 … of column c's 128-byte row from slot sl's 32 rows of A
+    constexpr int NCH = 8 / NSLOT;
+    auto column = [&](const float* src, int c, uint4 (&v)[NCH]) {
+#pragma unroll
+      for (int ch = 0; ch < NCH; ++ch) {
+        if constexpr (PREC == 2) {  // K = 16ch … 16ch + 15 as e4m3
+          const float* r = src + (size_t)(16 * ch) * TN + c;
+          v[ch] = make_uint4(pack_e4m3x4(r[0 * TN] * as, r[1 * TN] * as, r[2 * TN] * as, r[3 * TN] * as),
+                             pack_e4m3x4(r[4 * TN] * as, r[5 * TN] * as, r[6 * TN] * as, r[7 * TN] * as),
+                             pack_e4m3x4(r[8 * TN] * as, r[9 * TN] * as, r[10 * TN] * as, r[11 * TN] * as),
+                             pack_e4m3x4(r[12 * TN] * as, r[13 * TN] * as, r[14 * TN] * as, r[15 * TN] * as));
+        } else if constexpr (PREC == 1) {  // K = 8ch … 8ch + 7 as bf16
+          const float* r = src + (size_t)(8 * ch) * TN + c;
+          v[ch] = make_uint4(pack_bf16x2(r[0 * TN], r[1 * TN]), pack_bf16x2(r[2 * TN], r[3 * TN]),
+                             pack_bf16x2(r[4 * TN], r[5 * TN]), pack_bf16x2(r[6 * TN], r[7 * TN]));
+        } else {
+          const float* r = src + (size_t)(4 * ch) * TN + c;
+          v[ch] = make_uint4(to_tf32(r[0 * TN]), to_tf32(r[1 * TN]), to_tf32(r[2 * TN]), to_tf32(r[3 * TN]));
+        }
+      }
+    };
+    auto store = [&](unsigned char* dstA, int c, int sl, const uint4 (&v)[NCH]) {
+      unsigned char* row = dstA + (c >> 3) * 1024 + (c & 7) * 128;
+#pragma unroll
+      for (int ch = 0; ch < NCH; ++ch) *reinterpret_cast<uint4*>(row + (((NCH * sl + ch) ^ (c & 7)) << 4)) = v[ch];
+    };
     bool stop = false;
     for (int kb = 0; kb < nkb && !stop; ++kb) {
       const int s = kb % NSTAGE;
-      uint4 v[8];  // the column's 128-byte row, in 16-byte chunks of K
+      unsigned char* dstA = base + (size_t)s * kStageBytes + C::SBytes;
+      auto wait_stage = [&]() {
+        if (kb < NSTAGE || mbar_wait(&empty[s], ((uint32_t)(kb / NSTAGE) & 1u) ^ 1u, kWaitLimitNs)) return true;
+        atomicExch(&g_gauss_tc_error, MIHS_ERR_TIMEOUT);
+        return false;
+      };
+      uint4 early[EARLY ? NSLOT : 1][NCH];
+      if (!EARLY && !wait_stage()) break;
 #pragma unroll
       for (int sl = 0; sl < NSLOT; ++sl) {
         const int j = kb * NSLOT + sl;
@@ -374,47 +413,31 @@ gauss_tc_kernel(const __grid_constant__ CUtensorMap tmap_a, const GaussTcArgs a)
           stop = true;
           break;
         }
-        const float* src = reinterpret_cast<const float*>(stg + (size_t)q * kABytes) + c;  // [32 rows][256 cols]
-        if constexpr (PREC == 2) {
-          // 16-byte chunk ch = 2·sl + hh holds K = 16ch … 16ch + 15 as e4m3
-#pragma unroll
-          for (int hh = 0; hh < 2; ++hh) {
-            const float* r = src + (size_t)(16 * hh) * TN;
-            v[2 * sl + hh] = make_uint4(
-                pack_e4m3x4(r[0 * TN] * as, r[1 * TN] * as, r[2 * TN] * as, r[3 * TN] * as),
-                pack_e4m3x4(r[4 * TN] * as, r[5 * TN] * as, r[6 * TN] * as, r[7 * TN] * as),
-                pack_e4m3x4(r[8 * TN] * as, r[9 * TN] * as, r[10 * TN] * as, r[11 * TN] * as),
-                pack_e4m3x4(r[12 * TN] * as, r[13 * TN] * as, r[14 * TN] * as, r[15 * TN] * as));
-          }
-        } else if constexpr (PREC == 1) {
-          // 16-byte chunk ch = 4·sl + cc holds K = 8ch … 8ch + 7 as bf16
-#pragma unroll
-          for (int cc = 0; cc < 4; ++cc) {
-            const float* r = src + (size_t)(8 * cc) * TN;
-            v[4 * sl + cc] = make_uint4(pack_bf16x2(r[0 * TN], r[1 * TN]), pack_bf16x2(r[2 * TN], r[3 * TN]),
-                                        pack_bf16x2(r[4 * TN], r[5 * TN]), pack_bf16x2(r[6 * TN], r[7 * TN]));
-          }
+        const float* src = reinterpret_cast<const float*>(stg + (size_t)q * kABytes);  // [32 rows][256 cols]
+        if constexpr (EARLY) {
+          column(src, tt, early[sl]);
         } else {
 #pragma unroll
-          for (int ch = 0; ch < TK / 4; ++ch)
-            v[ch] = make_uint4(to_tf32(src[(4 * ch + 0) * TN]), to_tf32(src[(4 * ch + 1) * TN]),
-                               to_tf32(src[(4 * ch + 2) * TN]), to_tf32(src[(4 * ch + 3) * TN]));
+          for (int h = 0; h < NCOL; ++h) {
+            uint4 v[NCH];
+            column(src, tt + kTrWarps * 32 * h, v);
+            store(dstA, tt + kTrWarps * 32 * h, sl, v);
+          }
         }
         __syncwarp();
         if (lane == 0) mbar_arrive(&stg_empty[q]);  // this warp's reads of the slot are done
       }
       if (stop) break;
-      if (kb >= NSTAGE && !mbar_wait(&empty[s], ((uint32_t)(kb / NSTAGE) & 1u) ^ 1u, kWaitLimitNs)) {
-        atomicExch(&g_gauss_tc_error, MIHS_ERR_TIMEOUT);
-        break;
-      }
-      unsigned char* row = base + (size_t)s * kStageBytes + C::SBytes + (c >> 3) * 1024 + (c & 7) * 128;
+      if constexpr (EARLY) {
+        if (!wait_stage()) break;
 #pragma unroll
-      for (int ch = 0; ch < 8; ++ch) *reinterpret_cast<uint4*>(row + ((ch ^ (c & 7)) << 4)) = v[ch];
+        for (int sl = 0; sl < NSLOT; ++sl) store(dstA, tt, sl, early[sl]);
+      }
       fence_async_shared();  // generic-proxy writes → visible to the tensor core
       __syncwarp();
       if (lane == 0) mbar_arrive(&full[s]);
     }
+    __syncwarp();
   } else {
     // ------------------------------------------------------------ S generators
     // Item e of this block's slice: tile row g_lo + e/8, 16-byte chunk e mod 8
@@ -423,76 +446,82 @@ gauss_tc_kernel(const __grid_constant__ CUtensorMap tmap_a, const GaussTcArgs a)
     const int g = threadIdx.x - 64;
     const int nitems = (g_hi - g_lo) * 8;
     const uint32_t slice_off = (uint32_t)g_lo * 128u, slice_bytes = (uint32_t)(g_hi - g_lo) * 128u;
-    // The stage's entries are generated before the wait for the stage (a few
-    // hundred cycles that used to lie between the last MMA on it and the next).
+    // 16-byte chunk c of row gt of the stage at K = kbase
+    auto item = [&](int kbase, int gt, int c) {
+      const int gi = i0 + gt;
+      uint4 out = make_uint4(0u, 0u, 0u, 0u);
+      if constexpr (PREC == 2) {
+        // chunk c: K = kbase + 16c … + 15, four Philox counters
+        const int j0 = kbase + 16 * c;
+        if (gi < a.m && j0 < kb1) {
+          float z[16];
+#pragma unroll
+          for (int hh = 0; hh < 4; ++hh) {
+            const uint4 w = philox4x32_10(make_uint4((uint32_t)((j0 >> 2) + hh), (uint32_t)gi, kTagGaussian, 0u),
+                                          a.k0, a.k1);
+            const float2 za = box_muller_fast(w.x, w.y);
+            const float2 zb = box_muller_fast(w.z, w.w);
+            z[4 * hh + 0] = za.x;
+            z[4 * hh + 1] = za.y;
+            z[4 * hh + 2] = zb.x;
+            z[4 * hh + 3] = zb.y;
+          }
+#pragma unroll
+          for (int q = 0; q < 16; ++q)
+            if (j0 + q >= kb1) z[q] = 0.f;
+          out = make_uint4(pack_e4m3x4(z[0], z[1], z[2], z[3]), pack_e4m3x4(z[4], z[5], z[6], z[7]),
+                           pack_e4m3x4(z[8], z[9], z[10], z[11]), pack_e4m3x4(z[12], z[13], z[14], z[15]));
+        }
+      } else if constexpr (PREC == 1) {
+        // chunk c: K = kbase + 8c … + 7, two Philox counters
+        const int j0 = kbase + 8 * c;
+        if (gi < a.m && j0 < kb1) {
+          float z[8];
+#pragma unroll
+          for (int hh = 0; hh < 2; ++hh) {
+            const uint4 w = philox4x32_10(make_uint4((uint32_t)((j0 >> 2) + hh), (uint32_t)gi, kTagGaussian, 0u),
+                                          a.k0, a.k1);
+            const float2 za = box_muller_fast(w.x, w.y);
+            const float2 zb = box_muller_fast(w.z, w.w);
+            z[4 * hh + 0] = za.x;
+            z[4 * hh + 1] = za.y;
+            z[4 * hh + 2] = zb.x;
+            z[4 * hh + 3] = zb.y;
+          }
+#pragma unroll
+          for (int q = 0; q < 8; ++q)
+            if (j0 + q >= kb1) z[q] = 0.f;
+          out = make_uint4(pack_bf16x2(z[0], z[1]), pack_bf16x2(z[2], z[3]), pack_bf16x2(z[4], z[5]),
+                           pack_bf16x2(z[6], z[7]));
+        }
+      } else {
+        const int j0 = kbase + 4 * c;
+        if (gi < a.m && j0 < kb1) {
+          const uint4 w = philox4x32_10(make_uint4((uint32_t)(j0 >> 2), (uint32_t)gi, kTagGaussian, 0u), a.k0, a.k1);
+          const float2 za = box_muller_fast(w.x, w.y);
+          const float2 zb = box_muller_fast(w.z, w.w);
+          out = make_uint4(to_tf32(za.x), j0 + 1 < kb1 ? to_tf32(za.y) : 0u,
+                           j0 + 2 < kb1 ? to_tf32(zb.x) : 0u, j0 + 3 < kb1 ? to_tf32(zb.y) : 0u);
+        }
+      }
+      return out;
+    };
+    auto place = [&](int s, int gt, int c, const uint4& v) {
+      *reinterpret_cast<uint4*>(base + (size_t)s * kStageBytes + (size_t)gt * 128 + ((c ^ (gt & 7)) << 4)) = v;
+    };
     constexpr int NI = MROWS * 8 / (kGenWarps * 32);  // items per thread with one block per cluster
     for (int kb = 0; kb < nkb; ++kb) {
       const int s = kb % NSTAGE;
       const uint32_t ph = (uint32_t)(kb / NSTAGE) & 1u;
       const int kbase = kb0 + kb * KT;
-      uint4 items[NI];
+      uint4 early[EARLY ? NI : 1];
+      if constexpr (EARLY) {
 #pragma unroll
-      for (int i = 0; i < NI; ++i) {
-        const int e = g + i * kGenWarps * 32;
-        if (e >= nitems) break;
-        const int gt = g_lo + (e >> 3), c = e & 7;
-        const int gi = i0 + gt;
-        uint4 out = make_uint4(0u, 0u, 0u, 0u);
-        if constexpr (PREC == 2) {
-          // chunk c: K = kbase + 16c … + 15, four Philox counters
-          const int j0 = kbase + 16 * c;
-          if (gi < a.m && j0 < kb1) {
-            float z[16];
-#pragma unroll
-            for (int hh = 0; hh < 4; ++hh) {
-              const uint4 w = philox4x32_10(make_uint4((uint32_t)((j0 >> 2) + hh), (uint32_t)gi, kTagGaussian, 0u),
-                                            a.k0, a.k1);
-              const float2 za = box_muller_fast(w.x, w.y);
-              const float2 zb = box_muller_fast(w.z, w.w);
-              z[4 * hh + 0] = za.x;
-              z[4 * hh + 1] = za.y;
-              z[4 * hh + 2] = zb.x;
-              z[4 * hh + 3] = zb.y;
-            }
-#pragma unroll
-            for (int q = 0; q < 16; ++q)
-              if (j0 + q >= kb1) z[q] = 0.f;
-            out = make_uint4(pack_e4m3x4(z[0], z[1], z[2], z[3]), pack_e4m3x4(z[4], z[5], z[6], z[7]),
-                             pack_e4m3x4(z[8], z[9], z[10], z[11]), pack_e4m3x4(z[12], z[13], z[14], z[15]));
-          }
-        } else if constexpr (PREC == 1) {
-          // chunk c: K = kbase + 8c … + 7, two Philox counters
-          const int j0 = kbase + 8 * c;
-          if (gi < a.m && j0 < kb1) {
-            float z[8];
-#pragma unroll
-            for (int hh = 0; hh < 2; ++hh) {
-              const uint4 w = philox4x32_10(make_uint4((uint32_t)((j0 >> 2) + hh), (uint32_t)gi, kTagGaussian, 0u),
-                                            a.k0, a.k1);
-              const float2 za = box_muller_fast(w.x, w.y);
-              const float2 zb = box_muller_fast(w.z, w.w);
-              z[4 * hh + 0] = za.x;
-              z[4 * hh + 1] = za.y;
-              z[4 * hh + 2] = zb.x;
-              z[4 * hh + 3] = zb.y;
-            }
-#pragma unroll
-            for (int q = 0; q < 8; ++q)
-              if (j0 + q >= kb1) z[q] = 0.f;
-            out = make_uint4(pack_bf16x2(z[0], z[1]), pack_bf16x2(z[2], z[3]), pack_bf16x2(z[4], z[5]),
-                             pack_bf16x2(z[6], z[7]));
-          }
-        } else {
-          const int j0 = kbase + 4 * c;
-          if (gi < a.m && j0 < kb1) {
-            const uint4 w = philox4x32_10(make_uint4((uint32_t)(j0 >> 2), (uint32_t)gi, kTagGaussian, 0u), a.k0, a.k1);
-            const float2 za = box_muller_fast(w.x, w.y);
-            const float2 zb = box_muller_fast(w.z, w.w);
-            out = make_uint4(to_tf32(za.x), j0 + 1 < kb1 ? to_tf32(za.y) : 0u,
-                             j0 + 2 < kb1 ? to_tf32(zb.x) : 0u, j0 + 3 < kb1 ? to_tf32(zb.y) : 0u);
-          }
+        for (int i = 0; i < NI; ++i) {
+          const int e = g + i * kGenWarps * 32;
+          if (e >= nitems) break;
+          early[i] = item(kbase, g_lo + (e >> 3), e & 7);
         }
-        items[i] = out;
       }
       if (kb >= NSTAGE) {
         // One thread waits (bounded) and every generator takes its decision, so
@@ -504,20 +533,23 @@ gauss_tc_kernel(const __grid_constant__ CUtensorMap tmap_a, const GaussTcArgs a)
           break;
         }
       }
-      unsigned char* sS = base + (size_t)s * kStageBytes;
+      if constexpr (EARLY) {
 #pragma unroll
-      for (int i = 0; i < NI; ++i) {
-        const int e = g + i * kGenWarps * 32;
-        if (e >= nitems) break;
-        const int gt = g_lo + (e >> 3), c = e & 7;
-        *reinterpret_cast<uint4*>(sS + (size_t)gt * 128 + ((c ^ (gt & 7)) << 4)) = items[i];
+        for (int i = 0; i < NI; ++i) {
+          const int e = g + i * kGenWarps * 32;
+          if (e >= nitems) break;
+          place(s, g_lo + (e >> 3), e & 7, early[i]);
+        }
+      } else {
+        for (int e = g; e < nitems; e += kGenWarps * 32)
+          place(s, g_lo + (e >> 3), e & 7, item(kbase, g_lo + (e >> 3), e & 7));
       }
       fence_async_shared();            // the slice → visible to the async proxy (MMA, bulk copies)
       named_sync(1, kGenWarps * 32);   // every generator has written its part
       if (g == 0) {
         // This block's stage is complete once the peers' slices have landed.
         mbar_arrive_expect_tx(&full[s], (uint32_t)(MROWS * 128) - slice_bytes);
-        const uint32_t src = smem_u32(sS) + slice_off;
+        const uint32_t src = smem_u32(base + (size_t)s * kStageBytes) + slice_off;
         for (int p = 1; p < cn; ++p) {
           const uint32_t peer = (crank + (uint32_t)p) % (uint32_t)cn;
           bulk_copy_s2c(mapa(src, peer), src, slice_bytes, mapa(smem_u32(&full[s]), peer));
@@ -633,6 +665,20 @@ EncodeTiledFn encode_fn() {
   return fn;
 }
 
+// Whether a stage's operands are made ready before its last MMAs are done (see the
+// kernel), by type, sketch-row tiles per block, blocks per cluster and blocks along
+// the sketch rows.  µs late / early on both sides of the lines, 65536 rows of A, 588
+// rows of S unless stated: tf32 155 / 159 at 512 columns, 234 / 234 at 768, 271 / 254
+// at 1024, 444 / 439 at 1400, 598 / 610 at 1792; bf16 98 / 100 at 256, 116 / 115 at 512,
+// 165 / 151 at 1024, 350 / 336 at 1792; fp8 138 / 143 at 512, 189 / 189 at 1024 and with 200
+// rows 120 / 116, 226 / 232 at 1100 and with 200 rows 136 / 131.  One tile (64 rows):
+// tf32 52 / 51 at 512, 96 / 100 at 1100; bf16 50 / 49 at 600, 63 / 65 at 1100; fp8 85 / 83
+// at 600, 177 / 173 at 1792.
+bool early_operands(int prec, int mt, int cn, int tmb) {
+  if (mt == 1) return prec == 2 || cn <= 4;
+  return prec == 0 ? cn >= 3 && cn <= 6 : prec == 1 ? cn >= 2 : cn == 4 || (cn > 4 && tmb == 1);
+}
+
 }  // namespace
 
 bool gaussian_tc_available() { return encode_fn() != nullptr; }
@@ -648,14 +694,24 @@ int sketch_gaussian_tc(const float* A, int64_t n, int64_t d, int64_t lda, int64_
   }();
   const int tm = (int)((m + TM - 1) / TM);
   const int MT = (tm >= 2 && !force_mt1) ? 2 : 1;
-  const KernFn kern = prec == 2   ? (MT == 2 ? gauss_tc_kernel<2, 2> : gauss_tc_kernel<2, 1>)
-                     : prec == 1 ? (MT == 2 ? gauss_tc_kernel<1, 2> : gauss_tc_kernel<1, 1>)
-                                 : (MT == 2 ? gauss_tc_kernel<0, 2> : gauss_tc_kernel<0, 1>);
-  const size_t kSmemBytes = prec == 2   ? (MT == 2 ? TcCfg<2, 2>::Smem : TcCfg<2, 1>::Smem)
-                            : prec == 1 ? (MT == 2 ? TcCfg<1, 2>::Smem : TcCfg<1, 1>::Smem)
-                                        : (MT == 2 ? TcCfg<0, 2>::Smem : TcCfg<0, 1>::Smem);
-  const int KT = 32 << prec;
   const int tmb = (tm + MT - 1) / MT;  // blocks along the sketch rows
+  const int tn = (int)((d + TN - 1) / TN);
+  const bool early = early_operands(prec, MT, tn, tmb);
+  using Cfg = struct { KernFn kern; size_t smem; };
+  const auto pick = [early](auto early_kern, auto late_kern, size_t smem) {
+    return Cfg{early ? (KernFn)early_kern : (KernFn)late_kern, smem};
+  };
+  const Cfg cfg_k =
+      prec == 2   ? (MT == 2 ? pick(gauss_tc_kernel<2, 2, true>, gauss_tc_kernel<2, 2, false>, TcCfg<2, 2>::Smem)
+                             : pick(gauss_tc_kernel<2, 1, true>, gauss_tc_kernel<2, 1, false>, TcCfg<2, 1>::Smem))
+      : prec == 1 ? (MT == 2 ? pick(gauss_tc_kernel<1, 2, true>, gauss_tc_kernel<1, 2, false>, TcCfg<1, 2>::Smem)
+                             : pick(gauss_tc_kernel<1, 1, true>, gauss_tc_kernel<1, 1, false>, TcCfg<1, 1>::Smem))
+                  : (MT == 2 ? pick(gauss_tc_kernel<0, 2, true>, gauss_tc_kernel<0, 2, false>, TcCfg<0, 2>::Smem)
+                             : pick(gauss_tc_kernel<0, 1, true>, gauss_tc_kernel<0, 1, false>, TcCfg<0, 1>::Smem));
+  const KernFn kern = cfg_k.kern;
+  const size_t kSmemBytes = cfg_k.smem;
+  const int threads = tc_threads(early);
+  const int KT = 32 << prec;
   EncodeTiledFn enc = encode_fn();
   if (enc == nullptr) {
     set_error("gaussian sketch: cuTensorMapEncodeTiled unavailable");
@@ -673,7 +729,6 @@ int sketch_gaussian_tc(const float* A, int64_t n, int64_t d, int64_t lda, int64_
     set_error("gaussian sketch: cuTensorMapEncodeTiled failed (%d)", (int)r);
     return MIHS_ERR_UNSUPPORTED;
   }
-  const int tn = (int)((d + TN - 1) / TN);
   const int64_t kblocks = (n + KT - 1) / KT;
   MIHS_CUDA_TRY(cudaFuncSetAttribute((const void*)kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmemBytes));
   // One cluster per (sketch-row tile, K split) holds the tn column tiles.
@@ -687,7 +742,7 @@ int sketch_gaussian_tc(const float* A, int64_t n, int64_t d, int64_t lda, int64_
     attr[0].val.clusterDim.y = 1;
     attr[0].val.clusterDim.z = 1;
     cfg.gridDim = dim3((unsigned)tn, 1, 1);
-    cfg.blockDim = dim3(kThreads);
+    cfg.blockDim = dim3(threads);
     cfg.dynamicSmemBytes = kSmemBytes;
     cfg.attrs = attr;
     cfg.numAttrs = 1;
@@ -749,7 +804,7 @@ int sketch_gaussian_tc(const float* A, int64_t n, int64_t d, int64_t lda, int64_
     attr[0].val.clusterDim.y = 1;
     attr[0].val.clusterDim.z = 1;
     cfg.gridDim = dim3((unsigned)tn, (unsigned)tmb, (unsigned)KS);
-    cfg.blockDim = dim3(kThreads);
+    cfg.blockDim = dim3(threads);
     cfg.dynamicSmemBytes = kSmemBytes;
     cfg.stream = s;
     cfg.attrs = attr;

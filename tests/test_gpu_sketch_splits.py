@@ -6,6 +6,8 @@ import torch
 from oracle import mihs_oracle as o
 from paper_1912_03514_gb300 import mihs
 from paper_1912_03514_gb300 import workloads as W
+from tests import test_gpu_mixed as mixed
+from tests import test_gpu_parity as parity
 
 pytestmark = pytest.mark.gpu
 DEV = "cuda"
@@ -57,3 +59,13 @@ def test_srht_splits_are_exact(n, d, m):
                                    (6000, 16, 1241), (4100, 1023, 1249), (9001, 31, 1300), (20000, 2, 2481)])
 def test_srht_samples_past_the_registers(n, d, m):
     test_srht_splits_are_exact(n, d, m)
+
+
+# widths on both sides of those whose operands are made ready before their stage is free (clusters of four blocks),
+# one and two sketch-row tiles, stages fewer and more than the ring
+@pytest.mark.parametrize("n,d,m", [(3000, 768, 129), (3000, 769, 129), (60, 900, 40), (5000, 1023, 300),
+                                   (2049, 1024, 128), (2049, 1025, 257)])
+def test_gaussian_stage_orders(n, d, m):
+    parity.test_sketch_matches_oracle(o.GAUSSIAN, n, d, m)
+    mixed.test_gaussian_bf16_sketch_matches_oracle(n, d, m)
+    mixed.test_gaussian_fp8_sketch_matches_oracle(n, d, m)
