@@ -13,9 +13,15 @@
 // where its rows of each bucket begin without a global atomic, and the chunk
 // boundaries inside a bucket are known too (`start`).  At 262144×1024, m = 588:
 // 4 µs to count and 11 µs to scatter, where one global counter per bucket took
-// 34 and 35 µs (446 atomics on each of 588 words, ≈ 76 ns apiece).  Above
-// kHistMaxM buckets the counts outgrow a block and few rows meet on a counter:
-// that range keeps the global ones.
+// 34 and 35 µs (446 atomics on each of 588 words, ≈ 76 ns apiece).  With more
+// buckets every block reads more counts and fewer rows meet on a global counter,
+// which then is the cheaper: above kHistMaxM, or up to 4096 where a bucket has no
+// more than 64 rows (chunk counts / global counters: 262144×1024 to 2048 rows 202 /
+// 214 µs, to 4096 209 / 204, to 8192 243 / 214; 262144×64 to 3000 72 / 77,
+// 100000×200 to 3000 67 / 64).
+#include <algorithm>
+#include <type_traits>
+
 #include "internal.h"
 
 namespace mihs {
@@ -24,7 +30,7 @@ namespace {
 
 constexpr int kMaxChunks = 64;     // the scatter pass reads chunks × m counts in every block
 constexpr int kChunkRows = 2048;   // fewest rows worth a chunk
-constexpr int kHistMaxM = 8192;    // bucket counters of a chunk in shared memory (32 KB)
+constexpr int kHistMaxM = 2560;    // bucket counters of a chunk in shared memory (10 KB)
 constexpr int kSortThreads = 1024;
 constexpr int kGatherThreads = 256;
 constexpr int kSortCap = 8192;  // bucket entries sorted in shared memory
@@ -186,7 +192,16 @@ __device__ __forceinline__ float entry_sign(int e) { return e < 0 ? -1.f : 1.f; 
 // block per bucket, all 588 resident at once, ran as long as the fullest
 // bucket (180 µs); a bucket cut into chunk ranges (ks = 3 there) ends evenly:
 // 171 µs, 6.28 TB/s, 0.93 of the measured copy.
-template <int CT>
+//
+// RAGGED: the last group of a row is read whole too; its columns past the row are
+// the row's padding and never stored.  With a load of its own for it, 262144×1021
+// to 588 rows took 239 µs against 200, 100000×203 57 against 47.  More blocks per SM
+// read more rows at once and cost DRAM locality: this kernel needs 40 registers,
+// which leave six where matrices past L2 and whole rows per block take four (262144×1021
+// with six 222 µs); the other one's branch, never taken otherwise, makes it 63 and
+// so four (262144×1024 193 µs, without the branch and with six blocks 222).
+// (128 MB: about the L2.  37683×542 takes 45 µs with six, 48 with four.)
+template <int CT, bool WHOLE, bool RAGGED>
 __global__ void __launch_bounds__(kGatherThreads)
 cs_gather_kernel(const float* __restrict__ A, int n, int d, long long lda, const int* __restrict__ start,
                  const int* __restrict__ list, int m, int chunks, int ks, int slices, float* __restrict__ out,
@@ -194,11 +209,11 @@ cs_gather_kernel(const float* __restrict__ A, int n, int d, long long lda, const
   constexpr int RG = kGatherThreads / CT;
   __shared__ int keys[kSortCap];
   __shared__ float4 red[RG > 1 ? kGatherThreads : 1];
-  const long long unit = blockIdx.x;
-  const int slice = (int)(unit % slices);
-  const long long zh = unit / slices;
-  const int h = (int)(zh % m), z = (int)(zh / m);
-  const int z0 = (int)((long long)z * chunks / ks), z1 = (int)((long long)(z + 1) * chunks / ks);
+  // (32-bit arithmetic: buckets of a few rows end soon after it)
+  const unsigned zh = blockIdx.x / (unsigned)slices;
+  const int slice0 = (int)(blockIdx.x - zh * (unsigned)slices);
+  const int z = (int)(zh / (unsigned)m), h = (int)(zh - (unsigned)z * (unsigned)m);
+  const int z0 = z * chunks / ks, z1 = (z + 1) * chunks / ks;
   const int beg = start[(size_t)z0 * m + h];
   const int end = z1 < chunks ? start[(size_t)z1 * m + h] : (h + 1 < m ? start[h + 1] : n);
   const int cnt = end - beg;
@@ -228,60 +243,67 @@ cs_gather_kernel(const float* __restrict__ A, int n, int d, long long lda, const
     }
   }
   const int ct = threadIdx.x % CT, rg = threadIdx.x / CT;
-  const int col = 4 * (slice * CT + ct);
-  float4 acc = make_float4(0.f, 0.f, 0.f, 0.f);
-  if (col < d) {
-    const bool full = col + 4 <= d;
-    auto load = [&](int en) {
-      const float* row = A + (long long)entry_row(en) * lda + col;
-      if (full) return __ldcs(reinterpret_cast<const float4*>(row));
-      return make_float4(row[0], col + 1 < d ? row[1] : 0.f, col + 2 < d ? row[2] : 0.f, 0.f);
-    };
-    auto add = [&](int en, const float4& a) {
-      const float sg = entry_sign(en);
-      acc.x = fmaf(sg, a.x, acc.x);
-      acc.y = fmaf(sg, a.y, acc.y);
-      acc.z = fmaf(sg, a.z, acc.z);
-      acc.w = fmaf(sg, a.w, acc.w);
-    };
-    int e = rg;
-    for (; e + (kRowsInFlight - 1) * RG < cnt; e += kRowsInFlight * RG) {
-      int en[kRowsInFlight];
-      float4 a[kRowsInFlight];
+  auto sum_slice = [&](int slice) {
+    const int col = 4 * (slice * CT + ct);
+    float4 acc = make_float4(0.f, 0.f, 0.f, 0.f);
+    if (col < d) {
+      const bool full = col + 4 <= d;
+      auto load = [&](int en) {
+        const float* row = A + (long long)entry_row(en) * lda + col;
+        if (RAGGED || full) return __ldcs(reinterpret_cast<const float4*>(row));
+        return make_float4(row[0], col + 1 < d ? row[1] : 0.f, col + 2 < d ? row[2] : 0.f, 0.f);
+      };
+      auto add = [&](int en, const float4& a) {
+        const float sg = entry_sign(en);
+        acc.x = fmaf(sg, a.x, acc.x);
+        acc.y = fmaf(sg, a.y, acc.y);
+        acc.z = fmaf(sg, a.z, acc.z);
+        acc.w = fmaf(sg, a.w, acc.w);
+      };
+      int e = rg;
+      for (; e + (kRowsInFlight - 1) * RG < cnt; e += kRowsInFlight * RG) {
+        int en[kRowsInFlight];
+        float4 a[kRowsInFlight];
 #pragma unroll
-      for (int u = 0; u < kRowsInFlight; ++u) en[u] = sorted ? keys[e + u * RG] : list[beg + e + u * RG];
+        for (int u = 0; u < kRowsInFlight; ++u) en[u] = sorted ? keys[e + u * RG] : list[beg + e + u * RG];
 #pragma unroll
-      for (int u = 0; u < kRowsInFlight; ++u) a[u] = load(en[u]);
+        for (int u = 0; u < kRowsInFlight; ++u) a[u] = load(en[u]);
 #pragma unroll
-      for (int u = 0; u < kRowsInFlight; ++u) add(en[u], a[u]);
+        for (int u = 0; u < kRowsInFlight; ++u) add(en[u], a[u]);
+      }
+      for (; e < cnt; e += RG) {
+        const int en = sorted ? keys[e] : list[beg + e];
+        add(en, load(en));
+      }
     }
-    for (; e < cnt; e += RG) {
-      const int en = sorted ? keys[e] : list[beg + e];
-      add(en, load(en));
-    }
-  }
-  if constexpr (RG > 1) {
-    red[threadIdx.x] = acc;
-    __syncthreads();
-    if (rg != 0) return;
+    if constexpr (RG > 1) {
+      red[threadIdx.x] = acc;
+      __syncthreads();
+      if (rg != 0) return;
 #pragma unroll
-    for (int g = 1; g < RG; ++g) {
-      const float4 b = red[g * CT + ct];
-      acc.x += b.x;
-      acc.y += b.y;
-      acc.z += b.z;
-      acc.w += b.w;
+      for (int g = 1; g < RG; ++g) {
+        const float4 b = red[g * CT + ct];
+        acc.x += b.x;
+        acc.y += b.y;
+        acc.z += b.z;
+        acc.w += b.w;
+      }
     }
-  }
-  if (col >= d) return;
-  float* o = out + ((long long)z * m + h) * ldo + col;
-  if (col + 4 <= d && vec_out) {
-    *reinterpret_cast<float4*>(o) = acc;
+    if (col >= d) return;
+    float* o = out + ((long long)z * m + h) * ldo + col;
+    if (col + 4 <= d && vec_out) {
+      *reinterpret_cast<float4*>(o) = acc;
+    } else {
+      o[0] = acc.x;
+      if (col + 1 < d) o[1] = acc.y;
+      if (col + 2 < d) o[2] = acc.z;
+      if (col + 3 < d) o[3] = acc.w;
+    }
+  };
+  if constexpr (WHOLE) {  // all slices of the bucket (RG = 1: no barrier in a slice)
+    for (int slice = 0; slice * 4 * CT < d; ++slice) sum_slice(slice);
   } else {
-    o[0] = acc.x;
-    if (col + 1 < d) o[1] = acc.y;
-    if (col + 2 < d) o[2] = acc.z;
-    if (col + 3 < d) o[3] = acc.w;
+    sum_slice(slice0);
   }
 }
 
@@ -299,7 +321,7 @@ __global__ void cs_reduce_kernel(const float* __restrict__ part, int ks, int m, 
 
 int sketch_countsketch(const float* A, int64_t n, int64_t d, int64_t lda, int64_t m,
                        uint64_t seed, float* SA, int64_t ldsa, cudaStream_t s) {
-  const bool chunked = m <= kHistMaxM;
+  const bool chunked = m <= kHistMaxM || (m <= 4096 && n > 64 * m);
   int64_t chunks = 1, rows = n;
   if (chunked) {
     chunks = (n + kChunkRows - 1) / kChunkRows;
@@ -311,19 +333,34 @@ int sketch_countsketch(const float* A, int64_t n, int64_t d, int64_t lda, int64_
   const int64_t groups = (d + 3) / 4;
   int ct = 16;
   while (ct < 256 && ct < groups) ct *= 2;
-  const int slices = (int)((groups + ct - 1) / ct);
+  int slices = (int)((groups + ct - 1) / ct);
   // Chunk ranges per bucket: few and full buckets are cut so that two waves of
   // blocks (8 per SM) share the work and a block's entries can be sorted, as
-  // long as a thread still has eight rows to keep in flight.
-  const int64_t units = m * slices;
+  // long as a part still has 24 rows (32768×512 to 1024 rows: 47 µs cut into parts
+  // of 16, 41 whole), or, up to three blocks per SM, eight for each thread to keep
+  // in flight (8783×515 to 120 rows: 28 µs in parts of 15 to 18, 32 in parts of 24).
+  int64_t units = m * slices;
   const int64_t per_bucket = (n + m - 1) / m;
+  const int64_t least = kRowsInFlight * (kGatherThreads / ct);
   int64_t ks = (8LL * num_sms() + units - 1) / units;
-  const int64_t most = per_bucket / (kRowsInFlight * (kGatherThreads / ct));
+  int64_t most = per_bucket / (least > 24 ? least : 24);
+  const int64_t few = std::min<int64_t>((3LL * num_sms() + units - 1) / units, per_bucket / least);
+  if (most < few) most = few;
   if (ks > most) ks = most;
   const int64_t need = (per_bucket + kSortCap / 2 - 1) / (kSortCap / 2);
   if (ks < need) ks = need;
   if (ks > chunks) ks = chunks;
   if (ks < 1) ks = 1;
+  // of as many chunks each (five chunks in four parts take as long as in three)
+  const int64_t even = (chunks + chunks / ks - 1) / (chunks / ks);
+  if (even <= per_bucket / least) ks = even > ks ? even : ks;
+  // Buckets enough for two waves by themselves: a block sorts its bucket once for
+  // all slices of the row (50000×1500 to 20000 rows: 187 µs against 238).
+  const bool whole = slices > 1 && m * ks >= 16LL * num_sms();
+  if (whole) {
+    units = m;
+    slices = 1;
+  }
 
   StreamScratch scratch;
   const int64_t dp = round_up(d, 4);
@@ -362,12 +399,20 @@ int sketch_countsketch(const float* A, int64_t n, int64_t d, int64_t lda, int64_
   const long long ldo = ks > 1 ? (long long)dp : (long long)ldsa;
   const int vec_out = ldo % 4 == 0 && (reinterpret_cast<uintptr_t>(out) & 15u) == 0;
   const unsigned grid = (unsigned)(units * ks);
-  auto kern = ct == 256   ? cs_gather_kernel<256>
-              : ct == 128 ? cs_gather_kernel<128>
-              : ct == 64  ? cs_gather_kernel<64>
-              : ct == 32  ? cs_gather_kernel<32>
-                          : cs_gather_kernel<16>;
-  kern<<<grid, kGatherThreads, 0, s>>>(A, (int)n, (int)d, (long long)lda, start, list, (int)m, (int)chunks, (int)ks,
+  auto pick = [&](auto ragged) {
+    constexpr bool R = decltype(ragged)::value;
+    return whole       ? cs_gather_kernel<256, true, R>
+           : ct == 256 ? cs_gather_kernel<256, false, R>
+           : ct == 128 ? cs_gather_kernel<128, false, R>
+           : ct == 64  ? cs_gather_kernel<64, false, R>
+           : ct == 32  ? cs_gather_kernel<32, false, R>
+                       : cs_gather_kernel<16, false, R>;
+  };
+  const bool ragged = d % 4 != 0;
+  auto kern = ragged ? pick(std::true_type{}) : pick(std::false_type{});
+  // (16 KB more than the sort's 32 leave four blocks per SM)
+  const size_t idle = ragged && ct == 256 && n * lda * 4 > (128LL << 20) ? 16384 : 0;
+  kern<<<grid, kGatherThreads, idle, s>>>(A, (int)n, (int)d, (long long)lda, start, list, (int)m, (int)chunks, (int)ks,
                                        slices, out, ldo, vec_out);
   MIHS_CHECK_LAUNCH();
   count_launch();

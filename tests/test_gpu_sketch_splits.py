@@ -61,6 +61,14 @@ def test_srht_samples_past_the_registers(n, d, m):
     test_srht_splits_are_exact(n, d, m)
 
 
+# n, d, m: the most buckets that the chunk counters hold and the first past them, buckets that a block walks in several
+# slices after sorting them once, with a ragged last column group, and rows too few to cut a bucket
+@pytest.mark.parametrize("n,d,m", [(30000, 70, 2048), (30000, 70, 2049), (9000, 1501, 4000), (5000, 2047, 2500),
+                                   (32768, 512, 1024), (60000, 1030, 1300), (8192, 3, 8192)])
+def test_countsketch_many_buckets(n, d, m):
+    test_countsketch_splits_are_exact(n, d, m)
+
+
 # widths on both sides of those whose operands are made ready before their stage is free (clusters of four blocks),
 # one and two sketch-row tiles, stages fewer and more than the ring
 @pytest.mark.parametrize("n,d,m", [(3000, 768, 129), (3000, 769, 129), (60, 900, 40), (5000, 1023, 300),
