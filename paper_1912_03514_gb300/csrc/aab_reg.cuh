@@ -1,7 +1,9 @@
 // AAb_Solver (Algorithm 5, Section 3.6) as one thread-block cluster with SA in
 // registers, fused with the heavy-ball step of Eq. mihs1 and the stop test of
-// Algorithm 1: the form for every sketch that the registers of up to 16
-// blocks hold (m·d ≲ 650 K elements: 588 × 1024 takes 16 blocks).
+// Algorithm 1, for one λ or for a path (one cluster per λ): the form for every
+// sketch that the registers of up to 16 blocks hold.  Rows are padded to 256,
+// 512, 1024 or 2048 columns, of which those registers take 2560, 1280, 640 or
+// 256 (588 × 1024 takes 16 blocks).
 //
 // A pass is a chain of dependent steps (a product with SA, one with SAᵀ, two
 // norms), so what bounds it is the length of that chain, not any throughput.
