@@ -351,9 +351,12 @@ int sketch_countsketch(const float* A, int64_t n, int64_t d, int64_t lda, int64_
   if (ks < need) ks = need;
   if (ks > chunks) ks = chunks;
   if (ks < 1) ks = 1;
-  // of as many chunks each (five chunks in four parts take as long as in three)
+  // of as many chunks each (five chunks in four parts take as long as in three), but
+  // within the two waves: past them blocks that end early make room for the next, and
+  // more parts only cost (158618×256 to 32 rows: 38 uneven parts 58 µs, 64 even ones 66;
+  // 120000×256 to 64 rows, 19 and 20: 49.5 and 51.4).
   const int64_t even = (chunks + chunks / ks - 1) / (chunks / ks);
-  if (even <= per_bucket / least) ks = even > ks ? even : ks;
+  if (even > ks && even <= per_bucket / least && units * even <= 8LL * num_sms()) ks = even;
   // Buckets enough for two waves by themselves: a block sorts its bucket once for
   // all slices of the row (50000×1500 to 20000 rows: 187 µs against 238).
   const bool whole = slices > 1 && m * ks >= 16LL * num_sms();

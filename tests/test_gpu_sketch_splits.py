@@ -77,3 +77,10 @@ def test_gaussian_stage_orders(n, d, m):
     parity.test_sketch_matches_oracle(o.GAUSSIAN, n, d, m)
     mixed.test_gaussian_bf16_sketch_matches_oracle(n, d, m)
     mixed.test_gaussian_fp8_sketch_matches_oracle(n, d, m)
+
+
+# few buckets in many parts: parts of even and of uneven numbers of chunks, at and past two waves of blocks
+@pytest.mark.parametrize("n,d,m", [(131072, 17, 31), (131072, 64, 32), (131072, 33, 39), (81920, 256, 30), (81920, 130, 32),
+                                   (10240, 260, 97), (10241, 1027, 100), (131073, 4, 1)])
+def test_countsketch_few_buckets(n, d, m):
+    test_countsketch_splits_are_exact(n, d, m)
