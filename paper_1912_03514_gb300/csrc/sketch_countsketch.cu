@@ -195,12 +195,12 @@ __device__ __forceinline__ float entry_sign(int e) { return e < 0 ? -1.f : 1.f; 
 //
 // RAGGED: the last group of a row is read whole too; its columns past the row are
 // the row's padding and never stored.  With a load of its own for it, 262144×1021
-// to 588 rows took 239 µs against 200, 100000×203 57 against 47.  More blocks per SM
-// read more rows at once and cost DRAM locality: this kernel needs 40 registers,
-// which leave six where matrices past L2 and whole rows per block take four (262144×1021
-// with six 222 µs); the other one's branch, never taken otherwise, makes it 63 and
-// so four (262144×1024 193 µs, without the branch and with six blocks 222).
-// (128 MB: about the L2.  37683×542 takes 45 µs with six, 48 with four.)
+// to 588 rows took 239 µs against 200, 100000×203 57 against 47.  That load costs
+// little where the row's last warp holds few groups, see the launch.  More blocks per
+// SM read more rows at once and cost DRAM locality: this kernel needs 40 registers,
+// which leave six where wide rows take four (262144×1021 with six 222 µs); the other
+// one's branch, never taken otherwise, makes it 63 and so four (262144×1024 193 µs,
+// without the branch and with six blocks 222).
 template <int CT, bool WHOLE, bool RAGGED>
 __global__ void __launch_bounds__(kGatherThreads)
 cs_gather_kernel(const float* __restrict__ A, int n, int d, long long lda, const int* __restrict__ start,
@@ -411,10 +411,21 @@ int sketch_countsketch(const float* A, int64_t n, int64_t d, int64_t lda, int64_
            : ct == 32  ? cs_gather_kernel<32, false, R>
                        : cs_gather_kernel<16, false, R>;
   };
-  const bool ragged = d % 4 != 0;
+  // A load of its own for the last group is the better where the last warp of a row of
+  // more than 256 columns holds three groups or fewer: 668734×389 to 120 rows 238 µs
+  // against 296 read whole, 504123×517 to 502 265 against 287, 402061×650 254 against 282;
+  // with five and more, and in narrower rows, it is not (66971×545 to 502 72 against 63),
+  // nor where a block that walks all slices comes to these groups as a slice of their own
+  // (152409×1030 to 3000 rows 204 against 183).
+  const int64_t last = groups % 32;
+  const bool alone = whole && groups % ct == last;
+  const bool ragged = d % 4 != 0 && (groups <= 64 || last == 0 || last > 3 || alone);
   auto kern = ragged ? pick(std::true_type{}) : pick(std::false_type{});
-  // (16 KB more than the sort's 32 leave four blocks per SM)
-  const size_t idle = ragged && ct == 256 && n * lda * 4 > (128LL << 20) ? 16384 : 0;
+  // (16 KB more than the sort's 32 leave four blocks per SM.  Six / four: 481882×542 to
+  // 502 rows 266 / 289 µs, 51545×710 59 / 60, 368179×710 272 / 242, 24614×850 45 / 43,
+  // 307680×850 262 / 221.)
+  const int64_t four_from = groups > 192 ? 64 : groups > 150 ? 256 : INT64_MAX >> 20;
+  const size_t idle = ragged && ct == 256 && n * lda * 4 > (four_from << 20) ? 16384 : 0;
   kern<<<grid, kGatherThreads, idle, s>>>(A, (int)n, (int)d, (long long)lda, start, list, (int)m, (int)chunks, (int)ks,
                                        slices, out, ldo, vec_out);
   MIHS_CHECK_LAUNCH();

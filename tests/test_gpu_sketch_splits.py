@@ -84,3 +84,11 @@ def test_gaussian_stage_orders(n, d, m):
                                    (10240, 260, 97), (10241, 1027, 100), (131073, 4, 1)])
 def test_countsketch_few_buckets(n, d, m):
     test_countsketch_splits_are_exact(n, d, m)
+
+
+# ragged rows whose last warp holds three column groups and four, of more than 256 columns and fewer, a last slice of
+# one and of two groups in blocks that walk all slices and that do not, a matrix that takes four blocks per SM
+@pytest.mark.parametrize("n,d,m", [(5000, 139, 100), (5000, 267, 100), (5000, 271, 100), (9000, 517, 502), (9000, 525, 502),
+                                   (9000, 1025, 2500), (9000, 1030, 40), (20700, 815, 90)])
+def test_countsketch_last_groups(n, d, m):
+    test_countsketch_splits_are_exact(n, d, m)
